@@ -269,9 +269,11 @@ __global__ void __launch_bounds__(256) k3_sweep(Args3 a) {
                 out.x = n.phi;
                 ao0 += n.dE;
                 if (edge[0] || edge[1] || edge[2]) {
-                    float cn, sn;
-                    final_cs(n, C0, S0, cn, sn);
-                    const float dc = cn - n.co, ds = sn - n.so;
+                    float co, so, ca, sa, cn, sn;
+                    __sincosf(a.m.q * ph.x, &so, &co);
+                    __sincosf(a.m.q * n.mid, &sa, &ca);
+                    final_cs(n.refl, ca, sa, C0, S0, cn, sn);
+                    const float dc = cn - co, ds = sn - so;
 #pragma unroll
                     for (int k = 0; k < 3; ++k)
                         if (edge[k]) {
@@ -286,9 +288,11 @@ __global__ void __launch_bounds__(256) k3_sweep(Args3 a) {
                 out.y = n.phi;
                 ao1 += n.dE;
                 if (edge[0] || edge[1] || edge[2]) {
-                    float cn, sn;
-                    final_cs(n, C1, S1, cn, sn);
-                    const float dc = cn - n.co, ds = sn - n.so;
+                    float co, so, ca, sa, cn, sn;
+                    __sincosf(a.m.q * ph.y, &so, &co);
+                    __sincosf(a.m.q * n.mid, &sa, &ca);
+                    final_cs(n.refl, ca, sa, C1, S1, cn, sn);
+                    const float dc = cn - co, ds = sn - so;
 #pragma unroll
                     for (int k = 0; k < 3; ++k)
                         if (edge[k]) {

@@ -58,7 +58,7 @@ struct mpr_ctx {
     float* values = nullptr;
     uint8_t* mask = nullptr;
     float* dang = nullptr;
-    uint2* list[2] = {nullptr, nullptr};
+    uint4* list[2] = {nullptr, nullptr};
     int32_t* start[2] = {nullptr, nullptr};
     int32_t* split[2] = {nullptr, nullptr};
     double* Es = nullptr;
@@ -82,7 +82,7 @@ struct mpr_ctx {
     double* curve_e = nullptr;
     int curve_n = 0;
     float* T_site = nullptr;     // [H*W] site temperatures (SST), allocated on first use
-    float* beta_site = nullptr;  // [H*W] 1 / T_site
+    float* beta_site = nullptr;  // [2][H][Wh] 1 / T_site
     int sst = 0;                 // 1: realizations use the site temperatures
     double* msum = nullptr;      // [4][nblk] sums of E, E^2, E E_right, E E_down
     double* mom = nullptr;       // [4][nblk] moments of the last energy-moment run
@@ -105,8 +105,9 @@ struct mpr_ctx {
     int t = 0;
     int batch_open = 0;
     int storage = 0;             // element type of the batch state (an mpr_storage)
-    void* ang = nullptr;
-    size_t ang_cap = 0;          // bytes
+    void* ang_mem = nullptr;     // the state's allocation, with a guard on both sides
+    void* ang = nullptr;         // the state
+    size_t ang_cap = 0;          // bytes of ang_mem
     double* eacc = nullptr;
     double* ecur = nullptr;      // [nblk][Rp] current E_b of every (block, realization)
     double* ecur0 = nullptr;     // [nblk][Rp] calibration: E_b of the start state
@@ -120,7 +121,7 @@ struct mpr_ctx {
     size_t blk_cap = 0, lane_cap = 0, work_cap = 0;
     Control* ctl = nullptr;      // device loop state
     Control* h_ctl = nullptr;    // pinned mirror
-    int grid_cache[2][3][4] = {};  // full grid of k_sweep by (G = 2 / 8, storage, form)
+    int grid_cache[3][4] = {};   // full grid of k_sweep by (storage, form)
     // The WINDOW stop rule's ring of e_b (allocated when the rule is chosen).
     double* whist = nullptr;
     size_t whist_cap = 0;          // elements
@@ -309,16 +310,19 @@ mpr_status ensure_batch(mpr_ctx* ctx, int lanes, int requested_group, int storag
     const int G = pick_group(lanes, requested_group);
     const int groups = (lanes + G - 1) / G;
     const int Rp = groups * G;
-    const size_t ang_need = (size_t)groups * 2 * g.H * g.Wh * G * storage_bytes(storage);
+    const size_t guard = (state_guard(g) * storage_bytes(storage) + 255) / 256 * 256;
+    const size_t ang_need =
+        (size_t)groups * 2 * g.H * g.Wh * G * storage_bytes(storage) + 2 * guard;
     if (ang_need > ctx->ang_cap) {
-        dfree(ctx, ctx->ang);
-        ctx->ang = nullptr;
+        dfree(ctx, ctx->ang_mem);
+        ctx->ang_mem = ctx->ang = nullptr;
         ctx->ang_cap = 0;
         uint8_t* p = nullptr;
         TRY(dalloc(ctx, &p, ang_need));
-        ctx->ang = p;
+        ctx->ang_mem = p;
         ctx->ang_cap = ang_need;
     }
+    ctx->ang = static_cast<uint8_t*>(ctx->ang_mem) + guard;
     const size_t blk_need = (size_t)g.nblk * Rp;
     if (blk_need > ctx->blk_cap) {
         for (void* p : {(void*)ctx->eacc, (void*)ctx->running, (void*)ctx->stop, (void*)ctx->sigma,
@@ -497,9 +501,9 @@ int sweep_form(mpr_ctx* ctx) {
 }
 
 int sweep_grid(mpr_ctx* ctx, int form) {
-    int& full = ctx->grid_cache[ctx->G == 2 ? 0 : 1][ctx->storage][form];
-    if (full == 0) full = ctx->n_sm * sweep_blocks_per_sm(ctx->G, ctx->storage, form);
-    const unsigned long long ipc = (unsigned long long)sweep_items_per_cta(ctx->G, form);
+    int& full = ctx->grid_cache[ctx->storage][form];
+    if (full == 0) full = ctx->n_sm * sweep_blocks_per_sm(ctx->storage, form);
+    const unsigned long long ipc = (unsigned long long)sweep_items_per_cta(form);
     // (bound is ~0 while unknown: round up without overflowing)
     const unsigned long long need = ctx->bound / ipc + (ctx->bound % ipc != 0 ? 1 : 0);
     return (int)std::max<unsigned long long>(1, std::min<unsigned long long>(full, need));
@@ -511,7 +515,7 @@ void launch_halfstep(mpr_ctx* ctx, const SweepArgs& a, int form) {
         launch_sweep_tile(a, ctx->storage, tile_grid(ctx), ctx->s);
         return;
     }
-    launch_sweep(a, ctx->G, ctx->storage, form, sweep_grid(ctx, form), ctx->s);
+    launch_sweep(a, ctx->storage, form, sweep_grid(ctx, form), ctx->s);
 }
 
 // Grid of the stop kernels: a thread per (item, lane) or per item, at most
@@ -595,7 +599,7 @@ mpr_status init_batch_state(mpr_ctx* ctx) {
     const int random = ctx->opt.init == MPR_INIT_RANDOM;
     for (int c = 0; c < 2; ++c) {
         launch_init(ctx->g, ctx->sl, ctx->list[c], ctx->n_gap[c], c, ctx->init_angle, ctx->ang,
-                    ctx->storage, ctx->G, ctx->Rp, random, ctx->rng, ctx->r_even, ctx->s);
+                    ctx->storage, ctx->Rp / 2, random, ctx->rng, ctx->r_even, ctx->s);
         CKL();
     }
     return MPR_OK;
@@ -722,8 +726,7 @@ mpr_status moments_run(mpr_ctx* ctx, uint32_t tag, bool restart, int n_eq, int n
         ctx->r_even = 0;
         TRY(ensure_batch(ctx, chains, ctx->opt.group, MPR_STORE_F32));
         ctx->R = chains;
-        launch_fill_samples(g, ctx->mask, ctx->dang, ctx->ang, MPR_STORE_F32, ctx->G,
-                            ctx->groups, ctx->s);
+        launch_fill_samples(g, ctx->mask, ctx->dang, ctx->ang, MPR_STORE_F32, ctx->Rp / 2, ctx->s);
         CKL();
         TRY(init_batch_state(ctx));
         ctx->chains_valid = true;
@@ -925,7 +928,7 @@ mpr_status calibration_iteration(mpr_ctx* ctx, double inv_count, cudaGraphCondit
                 e1 = get_event(ctx);
                 if (e0) cudaEventRecord(e0, ctx->s);
             }
-            if (warp_form) launch_sweep_cal(a, ctx->G, ctx->s, f.ctas ? &f : nullptr);
+            if (warp_form) launch_sweep_cal(a, ctx->s, f.ctas ? &f : nullptr);
             else launch_sweep_flat(a, ctx->G, ctx->n_gap[c], ctx->s, f.ctas ? &f : nullptr);
             CKL();
             if (e0 && e1) {
@@ -1478,7 +1481,7 @@ mpr_status create_impl(const mpr_options* opt_in, int H, int W, int lb,
         cudaMemcpyAsync(ctx->ngap, ng.data(), g.nblk * 4, cudaMemcpyHostToDevice, ctx->s) ||
         cudaMemcpyAsync(ctx->Nsp_cal, nsp_cal.data(), g.nblk * 4, cudaMemcpyHostToDevice, ctx->s))
         return bail(MPR_ECUDA);
-    launch_build_lists(g, ctx->d_of_block, ctx->mask, ctx->start[0], ctx->start[1], ctx->list[0],
+    launch_build_lists(g, ctx->sl, ctx->mask, ctx->start[0], ctx->start[1], ctx->list[0],
                        ctx->list[1], ctx->split[0], ctx->split[1], ctx->s);
     ++ctx->launches;
     if (cudaMemsetAsync(ctx->sum, 0, 2 * plane * sizeof(double), ctx->s) ||
@@ -1773,8 +1776,7 @@ mpr_status mpr_calibrate(mpr_ctx* ctx, float* block_T_out) {
     launch_cal_init(g.nblk, o.t_lo, o.t_hi, ctx->lo, ctx->hi, ctx->ebar, ctx->ctl, ctx->s);
     CKL();
     const double inv_count = 1.0 / ((double)o.n_meas * (double)chains);
-    launch_fill_samples(g, ctx->mask, ctx->dang, ctx->ang, MPR_STORE_F32, ctx->G, ctx->groups,
-                        ctx->s);
+    launch_fill_samples(g, ctx->mask, ctx->dang, ctx->ang, MPR_STORE_F32, ctx->Rp / 2, ctx->s);
     CKL();
     // auto and 1: graph; 2: persistent; 3: a launch per kernel from the host.
     bool fallback = o.cal_mode != 2;
@@ -1843,8 +1845,7 @@ mpr_status mpr_sim_begin(mpr_ctx* ctx, int32_t n) {
     k_fill_valid<<<(int)std::min<int64_t>((nbr + 255) / 256, 152 * 16), 256, 0, ctx->s>>>(
         ctx->running, nbr, ctx->Rp, ctx->r_off, ctx->R);
     CKL();
-    launch_fill_samples(ctx->g, ctx->mask, ctx->dang, ctx->ang, ctx->storage, ctx->G, ctx->groups,
-                        ctx->s);
+    launch_fill_samples(ctx->g, ctx->mask, ctx->dang, ctx->ang, ctx->storage, ctx->Rp / 2, ctx->s);
     CKL();
     TRY(init_batch_state(ctx));
     CK(cudaMemsetAsync(ctx->tcount, 0, (size_t)ctx->Rp * ctx->n_slices * sizeof(int32_t), ctx->s));
@@ -1884,8 +1885,7 @@ mpr_status mpr_sim_end(mpr_ctx* ctx) {
     ctx->err.clear();
     if (!ctx->batch_open) return fail(ctx, MPR_ESTATE, "no open batch (mpr_sim_begin)");
     for (int c = 0; c < 2; ++c) {
-        launch_accumulate(ctx->g, ctx->list[c], ctx->n_gap[c], c, ctx->ang, ctx->storage, ctx->G,
-                          ctx->groups,
+        launch_accumulate(ctx->g, ctx->list[c], ctx->n_gap[c], c, ctx->ang, ctx->storage,
                           ctx->r_off, ctx->R, ctx->sum, ctx->s);
         CKL();
     }
@@ -1940,7 +1940,7 @@ mpr_status mpr_sample_chains(mpr_ctx* ctx, int32_t n_chains, int32_t n_equil, in
         if (t <= n_equil) continue;
         for (int c = 0; c < 2 && st == MPR_OK; ++c) {
             launch_accumulate(ctx->g, ctx->list[c], ctx->n_gap[c], c, ctx->ang, ctx->storage,
-                              ctx->G, ctx->groups, ctx->r_off, ctx->R, ctx->sum, ctx->s);
+                          ctx->r_off, ctx->R, ctx->sum, ctx->s);
             ++ctx->launches;
             if (cudaPeekAtLastError() != cudaSuccess)
                 st = fail(ctx, MPR_ECUDA, "sample_chains: accumulate launch failed");
@@ -2114,7 +2114,7 @@ SimTailArgs tail_args(mpr_ctx* ctx) {
 
 mpr_status simulate_tail(mpr_ctx* ctx, bool* ran) {
     *ran = false;
-    const int per_sm = ctx->coop ? sim_tail_blocks_per_sm(ctx->G, ctx->storage) : 0;
+    const int per_sm = ctx->coop ? sim_tail_blocks_per_sm(ctx->storage) : 0;
     if (per_sm < 1) return MPR_OK;
     const mpr_options& o = ctx->opt;
     SimTailArgs a = tail_args(ctx);
@@ -2128,7 +2128,7 @@ mpr_status simulate_tail(mpr_ctx* ctx, bool* ran) {
     // units per warp at the switch): few CTAs make the grid barriers cheap.
     const unsigned long long want = std::max<unsigned long long>(8, ctx->bound / 32);
     const int grid = (int)std::min<unsigned long long>((unsigned long long)ctx->n_sm * per_sm, want);
-    const cudaError_t le = launch_sim_tail(a, ctx->G, ctx->storage, grid, ctx->s);
+    const cudaError_t le = launch_sim_tail(a, ctx->storage, grid, ctx->s);
     if (le != cudaSuccess) {
         cudaGetLastError();
         if (tp.e0) ctx->ev_pool.push_back(tp.e0);
@@ -2159,7 +2159,7 @@ mpr_status simulate_pair_tail(mpr_ctx* ctx) {
     const SimTailArgs a = tail_args(ctx);
     TailProfile tp;
     TRY(tail_profile_begin(ctx, tp));
-    const cudaError_t le = launch_pair_tail(a, ctx->G, ctx->storage, ctx->Rp / 2, ctx->s);
+    const cudaError_t le = launch_pair_tail(a, ctx->storage, ctx->Rp / 2, ctx->s);
     if (le != cudaSuccess) return fail(ctx, MPR_ECUDA, "stop tail: %s", cudaGetErrorString(le));
     ++ctx->launches;
     TRY(tail_profile_end(ctx, tp));
@@ -2272,7 +2272,7 @@ mpr_status mpr_get_state(mpr_ctx* ctx, int32_t r, float* angles) {
     if (r < 0 || r >= ctx->R) return fail(ctx, MPR_EINVAL, "r out of range");
     const size_t n = (size_t)ctx->g.H * ctx->g.W;
     if (!ctx->out_buf) TRY(dalloc(ctx, &ctx->out_buf, n));
-    launch_get_state(ctx->g, ctx->mask, ctx->dang, ctx->ang, ctx->storage, ctx->G, r + ctx->r_off,
+    launch_get_state(ctx->g, ctx->mask, ctx->dang, ctx->ang, ctx->storage, r + ctx->r_off,
                      ctx->out_buf, ctx->s);
     CKL();
     return copy_out(ctx, angles, ctx->out_buf, n * 4);
@@ -2286,7 +2286,7 @@ mpr_status mpr_set_state(mpr_ctx* ctx, int32_t r, const float* angles) {
     const size_t n = (size_t)ctx->g.H * ctx->g.W;
     if (!ctx->truth_buf) TRY(dalloc(ctx, &ctx->truth_buf, n));
     TRY(copy_in(ctx, ctx->truth_buf, angles, n * 4));
-    launch_set_state(ctx->g, ctx->mask, ctx->ang, ctx->storage, ctx->G, r + ctx->r_off,
+    launch_set_state(ctx->g, ctx->mask, ctx->ang, ctx->storage, r + ctx->r_off,
                      ctx->truth_buf, ctx->s);
     CKL();
     CK(cudaStreamSynchronize(ctx->s));
@@ -2368,7 +2368,6 @@ mpr_status mpr_block_energy(mpr_ctx* ctx, int32_t r, double* E) {
     double* d = nullptr;
     TRY(dalloc(ctx, &d, ctx->g.nblk));
     launch_block_energy(ctx->g, ctx->d_of_block, ctx->mask, ctx->dang, ctx->ang, ctx->storage,
-                        ctx->G,
                         r + ctx->r_off, ctx->opt.q, ctx->opt.J, d, ctx->s);
     mpr_status st = MPR_OK;
     if (cudaPeekAtLastError() != cudaSuccess) st = fail(ctx, MPR_ECUDA, "block energy launch failed");
@@ -2381,7 +2380,7 @@ mpr_status mpr_block_energy(mpr_ctx* ctx, int32_t r, double* E) {
 mpr_status ensure_site_buffers(mpr_ctx* ctx) {
     const size_t n = (size_t)ctx->g.H * ctx->g.W;
     if (!ctx->T_site) TRY(dalloc(ctx, &ctx->T_site, n));
-    if (!ctx->beta_site) TRY(dalloc(ctx, &ctx->beta_site, n));
+    if (!ctx->beta_site) TRY(dalloc(ctx, &ctx->beta_site, 2 * (size_t)ctx->g.H * ctx->g.Wh));
     return MPR_OK;
 }
 
@@ -2426,7 +2425,7 @@ mpr_status mpr_set_site_temperatures(mpr_ctx* ctx, const float* T_site) {
         if (!(v > 0.0f) || !std::isfinite(v)) return fail(ctx, MPR_EINVAL, "site temperatures must be > 0");
     TRY(ensure_site_buffers(ctx));
     CK(cudaMemcpyAsync(ctx->T_site, h.data(), n * 4, cudaMemcpyHostToDevice, ctx->s));
-    launch_site_beta((int64_t)n, ctx->T_site, ctx->beta_site, ctx->s);
+    launch_site_beta(ctx->g, ctx->T_site, ctx->beta_site, ctx->s);
     CKL();
     CK(cudaStreamSynchronize(ctx->s));
     ctx->sst = 1;

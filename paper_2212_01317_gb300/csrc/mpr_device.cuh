@@ -60,6 +60,16 @@ __device__ __forceinline__ float u01(uint32_t x) {
     return __uint_as_float(0x3F800000u | (x >> 9)) - 0.999999940395355224609375f;
 }
 
+// The same from two words at once: the shift and the exponent bits are one
+// funnel shift (0x3F800000 = 0x7F << 23), the subtraction is packed.
+__device__ __forceinline__ float2 u01_2(uint32_t x, uint32_t y) {
+    return __fadd2_rn(make_float2(__uint_as_float(__funnelshift_r(x, 0x7Fu, 9)),
+                                  __uint_as_float(__funnelshift_r(y, 0x7Fu, 9))),
+                      make_float2(-0.999999940395355224609375f, -0.999999940395355224609375f));
+}
+
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+
 // psi = atan2(S, C) for S >= 0, psi in [0, pi]: atan(t) = t P(t^2) on
 // t = min/max of (|C|, S) in [0, 1], then the octant is restored. P is a
 // degree-7 near-minimax fit (gen_atan_poly.py; |error| < 7e-8 on [0, 1]).
@@ -81,27 +91,76 @@ __device__ __forceinline__ float atan2_upper(float S, float C) {
     return (C < 0.0f) ? (3.14159265358979324f - a) : a;
 }
 
-// Outcome of one site update.
+// 1 / x and 2^x of the hardware (PTX rcp / ex2, denormals flushed: x is a sum
+// of cosines or sines here, never denormal, and 2^x is compared with numbers
+// of at least 2^-24).
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float ex2_approx(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// atan2_upper of two arguments, the polynomial in packed arithmetic.
+__device__ __forceinline__ float2 atan2_upper_2(float2 S, float2 C) {
+    const float ax = fabsf(C.x), ay = fabsf(C.y);
+    const float2 mn = make_float2(fminf(ax, S.x), fminf(ay, S.y));
+    const float2 t = __fmul2_rn(mn, make_float2(rcp_approx(fmaxf(ax, S.x)),
+                                                rcp_approx(fmaxf(ay, S.y))));
+    const float2 z = __fmul2_rn(t, t);
+    float2 p = both(-4.054566845e-03f);
+    p = __ffma2_rn(p, z, both(2.186295763e-02f));
+    p = __ffma2_rn(p, z, both(-5.591232702e-02f));
+    p = __ffma2_rn(p, z, both(9.642197192e-02f));
+    p = __ffma2_rn(p, z, both(-1.390862912e-01f));
+    p = __ffma2_rn(p, z, both(1.994656622e-01f));
+    p = __ffma2_rn(p, z, both(-3.332985938e-01f));
+    p = __ffma2_rn(p, z, both(9.999993443e-01f));
+    float2 a = __fmul2_rn(t, p);
+    const float2 h = __ffma2_rn(a, both(-1.0f), both(1.57079632679489662f));
+    a = make_float2(S.x > ax ? h.x : a.x, S.y > ay ? h.y : a.y);
+    const float2 g = __ffma2_rn(a, both(-1.0f), both(3.14159265358979324f));
+    return make_float2(C.x < 0.0f ? g.x : a.x, C.y < 0.0f ? g.y : a.y);
+}
+
+// Outcome of one site update: the new angle, the angle after the Metropolis
+// move, the energy change, and whether the over-relaxation was applied.
 struct SiteNew {
-    float phi;      // new angle
-    float dE;       // energy change of the Metropolis move (0 when rejected)
-    float co, so;   // cos, sin of q * old angle
-    float ca, sa;   // cos, sin of q * angle after the Metropolis move
-    bool refl;      // over-relaxation applied
+    float phi, mid, dE;
+    bool refl;
 };
 
-// cos / sin of q times the final angle: after a reflection,
-// q phi'' = 2 psi - q phi_a with cos 2psi = (C^2 - S^2)/R^2, sin 2psi = 2CS/R^2.
-__device__ __forceinline__ void final_cs(const SiteNew& n, float C, float S, float& c, float& s) {
-    if (n.refl) {
+// Outcome of a site's update in both realizations of a pair (.x, .y): the new
+// angles, the angles after the Metropolis move, the energy change, and whether
+// the over-relaxation was applied.
+struct PairNew {
+    float2 phi, mid, dE;
+    bool refl0, refl1;
+};
+
+__device__ __forceinline__ void sincos_2(float2 x, float2& s, float2& c) {
+    __sincosf(x.x, &s.x, &c.x);
+    __sincosf(x.y, &s.y, &c.y);
+}
+
+// cos / sin of q times the final angle from those of q phi_a after the
+// Metropolis move: after a reflection q phi'' = 2 psi - q phi_a with
+// cos 2psi = (C^2 - S^2)/R^2, sin 2psi = 2CS/R^2.
+__device__ __forceinline__ void final_cs(bool refl, float ca, float sa, float C, float S, float& c,
+                                         float& s) {
+    if (refl) {
         const float ir2 = __fdividef(1.0f, C * C + S * S);
         const float c2 = (C * C - S * S) * ir2;
         const float s2 = 2.0f * C * S * ir2;
-        c = c2 * n.ca + s2 * n.sa;
-        s = s2 * n.ca - c2 * n.sa;
+        c = c2 * ca + s2 * sa;
+        s = s2 * ca - c2 * sa;
     } else {
-        c = n.ca;
-        s = n.sa;
+        c = ca;
+        s = sa;
     }
 }
 

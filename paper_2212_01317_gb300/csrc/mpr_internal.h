@@ -2,14 +2,19 @@
 //
 // Device memory of one context (one field):
 //   dang   [2][H][Wh] float   sample angles per checkerboard colour (0 at gaps)
-//   list_c [n_gap_c]  uint2   gap sites of colour c, block-major, row-major
-//                             within a block: .x = y << 16 | x, .y = b << 10 | flags
+//   list_c [n_gap_c]  uint4   gap sites of colour c, block-major, row-major
+//                             within a block: .x = half index, .y = b << 10 | flags,
+//                             .z = random-stream site index, .w = left half index
 //   start_c[nblk+1]   int32   list_c segment of every block
-//   ang    [groups][2][H][Wh][G]  angles of the batch (FP32, FP16 or BF16):
-//                             realization r = group * G + lane lives in lane
-//                             r % G of group r / G; the FP32 form also holds
-//                             the sample angles there, the 16-bit forms read
-//                             samples from dang only
+//   ang    [Rp/2][2][H][Wh]   words of the batch's realization pairs: two angles
+//                             (FP32, FP16 or BF16) of realizations 2 p and
+//                             2 p + 1, a plane per pair and colour. Sample
+//                             sites hold their FP32 angle: twice (FP32), or as
+//                             the four bytes of the word (16-bit).
+//                             A row and two half-sites before and after the
+//                             state are readable (state_guard), so a site at
+//                             the grid's border may load a neighbour that does
+//                             not exist
 //   eacc   [nblk][Rp] double  per-sweep energy change of each block (Rp = groups * G)
 //   ecur   [nblk][Rp] double  current block energy E_b
 //   running[nblk][Rp] uint8   1 while block b of realization r still sweeps
@@ -41,6 +46,13 @@ constexpr int MAX_SIDE = 32768;
 struct Geom {
     int H, W, Wh, lb, nbx, nby, nblk;
 };
+
+// Elements before and after the batch state that a neighbour load may touch.
+__host__ __device__ inline size_t state_guard(const Geom& g) { return 2 * ((size_t)g.Wh + 2); }
+// Element offset of pair p's plane of colour c.
+__host__ __device__ inline size_t pair_plane(const Geom& g, int p, int c) {
+    return ((size_t)p * 2 + (size_t)c) * g.H * g.Wh * 2;
+}
 
 struct Rng {
     uint32_t key0, key1;
@@ -138,13 +150,13 @@ struct SweepArgs {
     Rng rng;                  // key0 (seed_lo); key1 comes from the slice table
     Slices sl;
     int colour;
-    const uint2* list;        // gap entries of this colour
+    const uint4* list;        // gap entries of this colour (gap_item)
     const int32_t* start;     // [nblk + 1]
     const int32_t* split;     // [nblk] end of each block's edge entries
-    void* ang;                // batch state [groups][2][H][Wh][G] (FP32, FP16 or BF16)
+    void* ang;                // batch state [Rp/2][2][H][Wh] words (FP32, FP16 or BF16)
     const float* dang;        // [2][H][Wh] FP32 sample angles (0 at gaps)
     const float* beta;        // [nblk] 1 / T_b
-    const float* beta_site;   // [H*W] 1 / T_i (site temperatures, Sec. 2.2.3) or nullptr
+    const float* beta_site;   // [2][H][Wh] 1 / T_i (site temperatures, Sec. 2.2.3) or nullptr
     const float* beta_odd;    // [nblk] 1 / T_b of odd lanes (trisection's second point) or nullptr
     const float* beta_pts;    // [n_pts][nblk] 1 / T of the k-point calibration (lane r takes
                               // point r mod n_pts) or nullptr
@@ -217,7 +229,7 @@ struct GridBarrier {
 // barriers; the barrier closing a sweep also advances the Control.
 struct SimTailArgs {
     SweepArgs sw;              // colour-independent sweep fields
-    const uint2* list[2];
+    const uint4* list[2];
     const int32_t* start[2];
     const int32_t* split[2];
     StopArgs st;
@@ -230,7 +242,7 @@ struct SimTailArgs {
 // The persistent calibration kernel's arguments.
 struct CalPersistArgs {
     SweepArgs sw;              // colour-independent sweep fields (ecur, ang, beta, ...)
-    const uint2* list[2];
+    const uint4* list[2];
     const int32_t* start[2];
     const int32_t* split[2];
     int64_t n_list[2];

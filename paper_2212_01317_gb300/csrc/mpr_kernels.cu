@@ -10,6 +10,7 @@
 //   predict  conditional mean and back-transform (Sec. 2.1, 3.2), Eqs. 3-4
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "mpr_device.cuh"
@@ -187,17 +188,18 @@ __global__ void k_scan_counts(const int32_t* __restrict__ cnt, int n, int32_t* _
 // belongs to a neighbouring block (block edge), then the others, each group
 // in row-major order. Keeping the edge sites together lets most warps of the
 // sweep skip the per-bond energy split.
-__global__ void k_build_lists(Geom g, const int32_t* __restrict__ of_block,
+__global__ void k_build_lists(Geom g, Slices sl,
                               const uint8_t* __restrict__ mask,
                               const int32_t* __restrict__ start0, const int32_t* __restrict__ start1,
-                              uint2* __restrict__ list0, uint2* __restrict__ list1,
+                              uint4* __restrict__ list0, uint4* __restrict__ list1,
                               int32_t* __restrict__ split0, int32_t* __restrict__ split1) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= g.nblk) return;
     // Neighbours across the block's left / right / upper / lower edge exist
     // only in the same slice; within the slice, absent sites have no bonds.
-    const BlockFrame fr = block_frame(g, of_block, warp);
+    const BlockFrame fr = block_frame(g, sl.of_block, warp);
+    const int4 rect = fr.slice >= 0 ? slice_rect(sl, fr.slice) : make_int4(0, 0, 0, 0);
     const int bw = fr.x1 - fr.x0, nsite = (fr.y1 - fr.y0) * bw;
     int o0 = start0[fr.b], o1 = start1[fr.b];
     for (int pass = 0; pass < 2; ++pass) {
@@ -214,7 +216,7 @@ __global__ void k_build_lists(Geom g, const int32_t* __restrict__ of_block,
             const unsigned m0 = __ballot_sync(0xffffffffu, take && c == 0);
             const unsigned m1 = __ballot_sync(0xffffffffu, take && c == 1);
             if (take) {
-                const uint2 e = gap_entry(g, mask, fr, y, x);
+                const uint4 e = gap_item(g, rect, mask, fr, y, x);
                 const unsigned below = (1u << lane) - 1u;
                 if (c == 0) list0[o0 + __popc(m0 & below)] = e;
                 else list1[o1 + __popc(m1 & below)] = e;
@@ -232,73 +234,67 @@ __global__ void k_build_lists(Geom g, const int32_t* __restrict__ of_block,
 // ------------------------------------------------------------------ init --
 // Sec. 3.3.3: every gap site starts from the sample mean angle of its block
 // (global sample mean when the block has no sample); random start (plain
-// MPR) draws 2*pi*u from the reserved tag 0xFFFF.
+// MPR) draws 2*pi*u from the reserved tag 0xFFFF. One thread per gap entry;
+// blockIdx.y takes the realization pairs.
 template <typename S>
-__global__ void k_init(Geom g, Slices sl, const uint2* __restrict__ list, int64_t n_list,
-                       int colour, const float* __restrict__ init_angle, S* __restrict__ ang, int G,
-                       int Rp, int random, Rng rng, uint32_t r_even) {
-    const int64_t total = n_list * Rp;
-    const size_t plane = (size_t)g.H * g.Wh;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = t / Rp;
-        const int r = (int)(t % Rp);
-        const uint2 en = list[e];
-        const int y = en.x >> 16, x = en.x & 0xffff;
+__global__ void k_init(Geom g, Slices sl, const uint4* __restrict__ list, int64_t n_list,
+                       int colour, const float* __restrict__ init_angle, S* __restrict__ ang,
+                       int n_pairs, int random, Rng rng, uint32_t r_even) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_list;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const uint4 en = list[e];
         const int b = en.y >> META_SHIFT;
-        float v = init_angle[b];
-        if (random) {
-            const uint32_t gr = r_even + (uint32_t)r;
-            const int s = sl.of_block[b];
-            uint32_t w[4];
-            philox4x32_10(local_index(sl.rect[s], y, x), 0u | (0xFFFFu << 16), gr >> 1, 0u,
-                          rng.key0, sl.key1[s], w);
-            v = kTwoPi * u01(w[(gr & 1u) * 2u]);
+        const uint32_t key1 = random ? sl.key1[sl.of_block[b]] : 0u;
+        float2 v = both(init_angle[b]);
+        for (int p = blockIdx.y; p < n_pairs; p += gridDim.y) {
+            if (random) {
+                uint32_t w[4];
+                philox4x32_10(en.z, 0u | (0xFFFFu << 16), (r_even >> 1) + (uint32_t)p, 0u,
+                              rng.key0, key1, w);
+                v = make_float2(kTwoPi * u01(w[0]), kTwoPi * u01(w[2]));
+            }
+            Store<S>::store2(ang + pair_plane(g, p, colour) + 2 * (size_t)en.x, v);
         }
-        const int grp = r / G, lane = r % G;
-        Store<S>::store1(
-            ang + (((size_t)(grp * 2 + colour) * plane) + (size_t)y * g.Wh + (x >> 1)) * G + lane, v);
     }
 }
 
-// Sample angles copied into every lane of the batch state, so that a
-// neighbour read is the same load whether the neighbour is a gap or a sample.
+// Sample angles copied into every realization pair's word of the batch state,
+// so that a neighbour read is the same load whether the neighbour is a gap or
+// a sample: twice in FP32, the FP32 angle's four bytes in the 16-bit forms.
+// W: the word; blockIdx.y takes the pairs.
+template <typename W>
 __global__ void k_fill_samples(Geom g, const uint8_t* __restrict__ mask,
-                               const float* __restrict__ dang, float* __restrict__ ang, int G,
-                               int groups) {
+                               const float* __restrict__ dang, W* __restrict__ ang, int n_pairs) {
     const int64_t n = (int64_t)g.H * g.W;
     const size_t plane = (size_t)g.H * g.Wh;
-    const int64_t total = n * groups;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t % n;
-        const int grp = (int)(t / n);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
         if (mask[i]) continue;
         const int y = (int)(i / g.W), x = (int)(i % g.W);
-        const int c = (x + y) & 1;
-        const size_t hs = (size_t)y * g.Wh + (x >> 1);
-        const float v = dang[(size_t)c * plane + hs];
-        float* dst = ang + ((size_t)(grp * 2 + c) * plane + hs) * G;
-        for (int l = 0; l < G; ++l) dst[l] = v;
+        const size_t at = hidx(g, (x + y) & 1, y, x);
+        const float v = dang[at];
+        W w;
+        if constexpr (sizeof(W) == 8) w = make_float2(v, v);
+        else w = __float_as_uint(v);
+        for (int p = blockIdx.y; p < n_pairs; p += gridDim.y) ang[(size_t)p * 2 * plane + at] = w;
     }
 }
 
 // ----------------------------------------------------------------- sweep --
 // One half-step of the batch over the worklist of running units (or every
 // unit). A unit is one realization pair of one block: u = b * npairs + p
-// with npairs = Rp / 2 and pair p = group * (G/2) + q, so a pair whose two
+// with npairs = Rp / 2, so a pair whose two
 // realizations have stopped costs nothing. WPU warps take a unit (1: one
 // warp per pair; 2, 4: the pair's entries split between them, for the few
 // units left at the end of a batch), 128 / (32 WPU) units per CTA.
-template <int G, typename S, int WPU>
+template <typename S, int WPU>
 __global__ void __launch_bounds__(128, 8) k_sweep(SweepArgs a) {
     grid_dep_launch();
     grid_dep_wait();
-    constexpr int NP = G / 2;
     const uint32_t t = a.t_fixed > 0 ? (uint32_t)a.t_fixed : a.ctl->t;
     const uint32_t ctr1 = t | (a.ctl->tag << 16);
     const uint32_t* work = a.work ? a.work + (size_t)(t & 1u) * a.work_stride : nullptr;
-    const int npairs = a.groups * NP;
+    const int npairs = a.Rp >> 1;
     constexpr int UPC = 4 / WPU;
     const int warp = threadIdx.x >> 5;
     const int slot = warp / WPU, cw = warp % WPU;
@@ -309,23 +305,21 @@ __global__ void __launch_bounds__(128, 8) k_sweep(SweepArgs a) {
     const int n_units = work ? (int)a.ctl->n_work[t & 1u] : a.g.nblk * npairs;
     for (int it = it0; it < n_units; it += gridDim.x * UPC) {
         if (it != it0) u = work ? (int)work[it] : it;
-        const int b = u / npairs, p = u - b * npairs;
-        const int grp = p / NP, q = p - grp * NP;
-        sweep_item<G, S>(a, b * a.groups + grp, q + NP * cw, NP * WPU, ctr1);
+        const int b = u / npairs;
+        sweep_item<S>(a, b, u - b * npairs, cw, WPU, ctr1);
     }
 }
 
 // The same half-step with two units per warp (sweep_item_half), eight per
 // CTA: for short per-block entry lists.
-template <int G, typename S>
+template <typename S>
 __global__ void __launch_bounds__(128, 8) k_sweep_half(SweepArgs a) {
     grid_dep_launch();
     grid_dep_wait();
-    constexpr int NP = G / 2;
     const uint32_t t = a.t_fixed > 0 ? (uint32_t)a.t_fixed : a.ctl->t;
     const uint32_t ctr1 = t | (a.ctl->tag << 16);
     const uint32_t* work = a.work ? a.work + (size_t)(t & 1u) * a.work_stride : nullptr;
-    const int npairs = a.groups * NP;
+    const int npairs = a.Rp >> 1;
     const int warp = threadIdx.x >> 5, half = (threadIdx.x >> 4) & 1;
     const int it0 = blockIdx.x * 8 + warp * 2 + half;
     int u = work ? (it0 < (int)a.work_stride ? (int)work[it0] : 0) : it0;
@@ -335,9 +329,8 @@ __global__ void __launch_bounds__(128, 8) k_sweep_half(SweepArgs a) {
         const int it = base + half;
         const bool have = it < n_units;
         if (it != it0) u = have ? (work ? (int)work[it] : it) : 0;
-        const int b = u / npairs, p = u - b * npairs;
-        const int grp = p / NP, q = p - grp * NP;
-        sweep_item_half<G, S>(a, b * a.groups + grp, q, have, ctr1);
+        const int b = u / npairs;
+        sweep_item_half<S>(a, b, u - b * npairs, have, ctr1);
     }
 }
 
@@ -398,7 +391,7 @@ __global__ void __launch_bounds__(kFlatThreads, 8) k_sweep_flat(SweepArgs a, int
 // setup (entry, random block, temperatures, block sums) weighs on every
 // update; the flat form stays for lists of a few waves, which it covers in
 // one latency chain.
-template <int G>
+template <bool kAll>
 __global__ void __launch_bounds__(128, 8) k_sweep_cal(SweepArgs a, FoldArgs f) {
     grid_dep_launch();
     grid_dep_wait();
@@ -407,29 +400,25 @@ __global__ void __launch_bounds__(128, 8) k_sweep_cal(SweepArgs a, FoldArgs f) {
         fold_block_energies<128>(f, (int)blockIdx.x - sweep_ctas);
         return;
     }
-    constexpr int NP = G / 2;
     const uint32_t t = a.t_fixed > 0 ? (uint32_t)a.t_fixed : a.ctl->t;
     const uint32_t ctr1 = t | (a.ctl->tag << 16);
-    const int npairs = a.groups * NP;
+    const int npairs = a.Rp >> 1;
     const int n_units = a.g.nblk * npairs;
     for (int u = blockIdx.x * 4 + (int)(threadIdx.x >> 5); u < n_units; u += sweep_ctas * 4) {
-        const int b = u / npairs, p = u - b * npairs;
-        const int grp = p / NP, q = p - grp * NP;
-        sweep_item<G, float, true>(a, b * a.groups + grp, q, NP, ctr1);
+        const int b = u / npairs;
+        sweep_item<float, true, kAll>(a, b, u - b * npairs, 0, 1, ctr1);
     }
 }
 
-template <int G, typename S>
-__global__ void __launch_bounds__(128) k_energy(SweepArgs a) {
+template <typename S>
+__global__ void __launch_bounds__(128) k_energy(SweepArgs a, int NP) {
     const int n_items = a.g.nblk * a.groups;
     for (int it = blockIdx.x; it < n_items; it += gridDim.x)
-        energy_item<G, S>(a, it, threadIdx.x >> 5, 4);
+        energy_item<S>(a, it / a.groups, it % a.groups, NP, threadIdx.x >> 5, 4);
 }
 
 template __global__ void k_sweep_flat<2>(SweepArgs, int64_t, FoldArgs);
 template __global__ void k_sweep_flat<8>(SweepArgs, int64_t, FoldArgs);
-template __global__ void k_sweep_cal<2>(SweepArgs, FoldArgs);
-template __global__ void k_sweep_cal<8>(SweepArgs, FoldArgs);
 
 // ------------------------------------------------------------------ stop --
 // es[b] = E_s,b / N_SP,b (0 without sample bonds) and inb[b] = 1 / N_b (0 for
@@ -760,19 +749,16 @@ __global__ void k_cal_update(int nblk, double inv_count, const double* __restric
 // --------------------------------------------------------------- predict --
 // Adds the batch's final angles of every gap site to the running sums.
 template <typename S>
-__global__ void k_accumulate(Geom g, const uint2* __restrict__ list, int64_t n_list, int colour,
-                             const S* __restrict__ ang, int G, int groups, int r_off, int R,
+__global__ void k_accumulate(Geom g, const uint4* __restrict__ list, int64_t n_list, int colour,
+                             const S* __restrict__ ang, int r_off, int R,
                              double* __restrict__ sum) {
     const size_t plane = (size_t)g.H * g.Wh;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_list;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const uint2 en = list[e];
-        const int y = en.x >> 16, x = en.x & 0xffff;
-        const size_t hs = (size_t)y * g.Wh + (x >> 1);
+        const size_t hs = list[e].x;
         double s = 0.0;
         for (int r = r_off; r < r_off + R; ++r) {
-            const int grp = r / G, lane = r % G;
-            s += (double)Store<S>::load1(ang + ((size_t)(grp * 2 + colour) * plane + hs) * G + lane);
+            s += (double)Store<S>::load1(ang + pair_plane(g, r >> 1, colour) + 2 * hs + (r & 1));
         }
         sum[(size_t)colour * plane + hs] += s;
     }
@@ -859,34 +845,31 @@ __global__ void k_predict(Geom g, Slices sl, const float* __restrict__ values,
 // ------------------------------------------------------- state access --
 template <typename S>
 __global__ void k_get_state(Geom g, const uint8_t* __restrict__ mask, const float* __restrict__ dang,
-                            const S* __restrict__ ang, int G, int r, float* __restrict__ out) {
+                            const S* __restrict__ ang, int r, float* __restrict__ out) {
     const int64_t n = (int64_t)g.H * g.W;
     const size_t plane = (size_t)g.H * g.Wh;
-    const int grp = r / G, lane = r % G;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int y = (int)(i / g.W), x = (int)(i % g.W);
         const int c = (x + y) & 1;
         const size_t hs = (size_t)y * g.Wh + (x >> 1);
         out[i] = mask[i] == MASK_GAP
-                     ? Store<S>::load1(ang + ((size_t)(grp * 2 + c) * plane + hs) * G + lane)
+                     ? Store<S>::load1(ang + pair_plane(g, r >> 1, c) + 2 * hs + (r & 1))
                      : dang[(size_t)c * plane + hs];
     }
 }
 
 template <typename S>
 __global__ void k_set_state(Geom g, const uint8_t* __restrict__ mask, S* __restrict__ ang,
-                            int G, int r, const float* __restrict__ in) {
+                            int r, const float* __restrict__ in) {
     const int64_t n = (int64_t)g.H * g.W;
-    const size_t plane = (size_t)g.H * g.Wh;
-    const int grp = r / G, lane = r % G;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (mask[i] != MASK_GAP) continue;
         const int y = (int)(i / g.W), x = (int)(i % g.W);
         const int c = (x + y) & 1;
         const size_t hs = (size_t)y * g.Wh + (x >> 1);
-        Store<S>::store1(ang + ((size_t)(grp * 2 + c) * plane + hs) * G + lane, in[i]);
+        Store<S>::store1(ang + pair_plane(g, r >> 1, c) + 2 * hs + (r & 1), in[i]);
     }
 }
 
@@ -894,18 +877,17 @@ __global__ void k_set_state(Geom g, const uint8_t* __restrict__ mask, S* __restr
 template <typename S>
 __global__ void k_block_energy(Geom g, const int32_t* __restrict__ of_block,
                                const uint8_t* __restrict__ mask,
-                               const float* __restrict__ dang, const S* __restrict__ ang, int G,
+                               const float* __restrict__ dang, const S* __restrict__ ang,
                                int r, double q, double J, double* __restrict__ E) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= g.nblk) return;
     const size_t plane = (size_t)g.H * g.Wh;
-    const int grp = r / G, ln = r % G;
     auto angle = [&](int y, int x) -> double {
         const int c = (x + y) & 1;
         const size_t hs = (size_t)y * g.Wh + (x >> 1);
         return mask[(int64_t)y * g.W + x] == MASK_GAP
-                   ? (double)Store<S>::load1(ang + ((size_t)(grp * 2 + c) * plane + hs) * G + ln)
+                   ? (double)Store<S>::load1(ang + pair_plane(g, r >> 1, c) + 2 * hs + (r & 1))
                    : (double)dang[(size_t)c * plane + hs];
     };
     // A bond exists between present sites of the same slice.
@@ -1062,19 +1044,28 @@ __global__ void k_sst_box(Geom g, Slices sl, const double* __restrict__ in,
     }
 }
 
-__global__ void k_site_beta(int64_t n, const float* __restrict__ Tf, float* __restrict__ beta) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        beta[i] = 1.0f / Tf[i];
+// Site beta in the sweep's half-lattice order.
+__device__ __forceinline__ void store_beta(const Geom& g, int64_t i, float t,
+                                           float* __restrict__ beta) {
+    const int y = (int)(i / g.W), x = (int)(i % g.W);
+    beta[hidx(g, (x + y) & 1, y, x)] = 1.0f / t;
 }
 
-__global__ void k_sst_beta(int64_t n, const double* __restrict__ Ts, float* __restrict__ Tf,
+__global__ void k_site_beta(Geom g, const float* __restrict__ Tf, float* __restrict__ beta) {
+    const int64_t n = (int64_t)g.H * g.W;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        store_beta(g, i, Tf[i], beta);
+}
+
+__global__ void k_sst_beta(Geom g, const double* __restrict__ Ts, float* __restrict__ Tf,
                            float* __restrict__ beta) {
+    const int64_t n = (int64_t)g.H * g.W;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float t = (float)Ts[i];
         Tf[i] = t;
-        beta[i] = 1.0f / t;
+        store_beta(g, i, t, beta);
     }
 }
 
@@ -1116,12 +1107,12 @@ void launch_scan(const int32_t* cnt, int n, int32_t* out, cudaStream_t s) {
     k_scan_counts<<<1, 1024, 0, s>>>(cnt, n, out);
 }
 
-void launch_build_lists(const Geom& g, const int32_t* of_block, const uint8_t* mask,
-                        const int32_t* start0, const int32_t* start1, uint2* list0, uint2* list1,
+void launch_build_lists(const Geom& g, const Slices& sl, const uint8_t* mask,
+                        const int32_t* start0, const int32_t* start1, uint4* list0, uint4* list1,
                         int32_t* split0, int32_t* split1, cudaStream_t s) {
     const int threads = 256;
     const int blocks = (int)(((int64_t)g.nblk * 32 + threads - 1) / threads);
-    k_build_lists<<<blocks, threads, 0, s>>>(g, of_block, mask, start0, start1, list0, list1,
+    k_build_lists<<<blocks, threads, 0, s>>>(g, sl, mask, start0, start1, list0, list1,
                                              split0, split1);
 }
 
@@ -1157,80 +1148,67 @@ template <typename F> void with_storage(int storage, F&& f) {
 }
 }  // namespace
 
-void launch_init(const Geom& g, const Slices& sl, const uint2* list, int64_t n_list, int colour,
-                 const float* init_angle, void* ang, int storage, int G, int Rp, int random,
+void launch_init(const Geom& g, const Slices& sl, const uint4* list, int64_t n_list, int colour,
+                 const float* init_angle, void* ang, int storage, int n_pairs, int random,
                  Rng rng, uint32_t r_even, cudaStream_t s) {
     if (n_list == 0) return;
+    // (a pair per blockIdx.y while that leaves a wave or less along x)
+    const int gx = grid_for(n_list, 256);
+    const dim3 grid((unsigned)gx, (unsigned)std::max(1, std::min(n_pairs, 152 * 16 / gx)));
     with_storage(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
-        k_init<S><<<grid_for(n_list * Rp, 256), 256, 0, s>>>(g, sl, list, n_list, colour,
-                                                            init_angle, static_cast<S*>(ang), G,
-                                                            Rp, random, rng, r_even);
+        k_init<S><<<grid, 256, 0, s>>>(g, sl, list, n_list, colour, init_angle,
+                                       static_cast<S*>(ang), n_pairs, random, rng, r_even);
     });
 }
 
 void launch_fill_samples(const Geom& g, const uint8_t* mask, const float* dang, void* ang,
-                         int storage, int G, int groups, cudaStream_t s) {
-    if (storage != 0) return;        // the 16-bit forms read samples from dang
-    k_fill_samples<<<grid_for((int64_t)g.H * g.W * groups, 256), 256, 0, s>>>(
-        g, mask, dang, static_cast<float*>(ang), G, groups);
+                         int storage, int n_pairs, cudaStream_t s) {
+    const int gx = grid_for((int64_t)g.H * g.W, 256);
+    const dim3 grid((unsigned)gx, (unsigned)std::max(1, std::min(n_pairs, 152 * 16 / gx)));
+    if (storage == 0)
+        k_fill_samples<<<grid, 256, 0, s>>>(g, mask, dang, static_cast<float2*>(ang), n_pairs);
+    else
+        k_fill_samples<<<grid, 256, 0, s>>>(g, mask, dang, static_cast<uint32_t*>(ang), n_pairs);
 }
 
 namespace {
 // The three forms of the realizations' half-step by warps per unit (one
 // realization pair of one block): form 0 one warp, form 1 two, form 2 four
 // (splitting the block's entries between them), in 128-thread CTAs.
-template <int G, typename S>
-void sweep_dispatch(const SweepArgs& a, int form, int grid, cudaStream_t s) {
-    if (form == 3) launch_pdl(k_sweep_half<G, S>, grid, 128, s, a);
-    else if (form == 2) launch_pdl(k_sweep<G, S, 4>, grid, 128, s, a);
-    else if (form == 1) launch_pdl(k_sweep<G, S, 2>, grid, 128, s, a);
-    else launch_pdl(k_sweep<G, S, 1>, grid, 128, s, a);
-}
-
-template <int G, typename S>
-int sweep_occupancy(int form) {
-    int n = 0;
-    if (form == 3) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep_half<G, S>, 128, 0);
-    else if (form == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<G, S, 4>, 128, 0);
-    else if (form == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<G, S, 2>, 128, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<G, S, 1>, 128, 0);
-    return n > 0 ? n : 1;
+template <typename S> auto sweep_kernel(int form) {
+    return form == 3 ? k_sweep_half<S>
+           : form == 2 ? k_sweep<S, 4>
+           : form == 1 ? k_sweep<S, 2>
+                       : k_sweep<S, 1>;
 }
 }  // namespace
 
-void launch_sweep(const SweepArgs& a, int G, int storage, int form, int grid, cudaStream_t s) {
+void launch_sweep(const SweepArgs& a, int storage, int form, int grid, cudaStream_t s) {
     with_storage(storage, [&](auto tag) {
-        using S = typename decltype(tag)::type;
-        if (G == 2) sweep_dispatch<2, S>(a, form, grid, s);
-        else sweep_dispatch<8, S>(a, form, grid, s);
+        launch_pdl(sweep_kernel<typename decltype(tag)::type>(form), grid, 128, s, a);
     });
 }
 
-int sweep_blocks_per_sm(int G, int storage, int form) {
-    int n = 1;
+int sweep_blocks_per_sm(int storage, int form) {
+    int n = 0;
     with_storage(storage, [&](auto tag) {
-        using S = typename decltype(tag)::type;
-        n = G == 2 ? sweep_occupancy<2, S>(form) : sweep_occupancy<8, S>(form);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &n, sweep_kernel<typename decltype(tag)::type>(form), 128, 0);
     });
-    return n;
+    return n > 0 ? n : 1;
 }
 
-int sweep_items_per_cta(int G, int form) {
-    (void)G;
-    return form == 3 ? 8 : 4 >> form;
-}
+int sweep_items_per_cta(int form) { return form == 3 ? 8 : 4 >> form; }
 
 void launch_energy(const SweepArgs& a, int G, int storage, int n_sm, cudaStream_t s) {
     with_storage(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
         // As many CTAs as fit on the GPU at once (the kernel loops over items).
         int per_sm = 0;
-        if (G == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_energy<2, S>, 128, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_energy<8, S>, 128, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_energy<S>, 128, 0);
         const int grid = n_sm * (per_sm > 0 ? per_sm : 8);
-        if (G == 2) k_energy<2, S><<<grid, 128, 0, s>>>(a);
-        else k_energy<8, S><<<grid, 128, 0, s>>>(a);
+        k_energy<S><<<grid, 128, 0, s>>>(a, G / 2);
     });
 }
 
@@ -1248,13 +1226,14 @@ void launch_sweep_flat(const SweepArgs& a, int G, int64_t n_list, cudaStream_t s
     else launch_pdl(k_sweep_flat<8>, grid, kFlatThreads, s, a, n_list, f);
 }
 
-void launch_sweep_cal(const SweepArgs& a, int G, cudaStream_t s, const FoldArgs* fold) {
+void launch_sweep_cal(const SweepArgs& a, cudaStream_t s, const FoldArgs* fold) {
     FoldArgs f{};
     if (fold) f = *fold;
-    const int64_t units = (int64_t)a.g.nblk * a.groups * (G / 2);
+    const int64_t units = (int64_t)a.g.nblk * (a.Rp >> 1);
     const dim3 grid((unsigned)((units + 3) / 4 + f.ctas));
-    if (G == 2) launch_pdl(k_sweep_cal<2>, grid, 128, s, a, f);
-    else launch_pdl(k_sweep_cal<8>, grid, 128, s, a, f);
+    // (an even number of lanes: both realizations of every pair run)
+    if (a.R == a.Rp) launch_pdl(k_sweep_cal<true>, grid, 128, s, a, f);
+    else launch_pdl(k_sweep_cal<false>, grid, 128, s, a, f);
 }
 
 // Lanes G.. Rp-1 of every block take the E_b of lane r mod G (all lanes hold
@@ -1390,14 +1369,14 @@ void launch_cal_update(int nblk, double inv_count, const double* es, const int32
                                                     ctl, n_bisect, cond);
 }
 
-void launch_accumulate(const Geom& g, const uint2* list, int64_t n_list, int colour,
-                       const void* ang, int storage, int G, int groups, int r_off, int R,
-                       double* sum, cudaStream_t s) {
+void launch_accumulate(const Geom& g, const uint4* list, int64_t n_list, int colour,
+                       const void* ang, int storage, int r_off, int R, double* sum,
+                       cudaStream_t s) {
     if (n_list == 0) return;
     with_storage(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
         k_accumulate<S><<<grid_for(n_list, 256), 256, 0, s>>>(
-            g, list, n_list, colour, static_cast<const S*>(ang), G, groups, r_off, R, sum);
+            g, list, n_list, colour, static_cast<const S*>(ang), r_off, R, sum);
     });
 }
 
@@ -1419,32 +1398,32 @@ void launch_predict(const Geom& g, const Slices& sl, const float* values, const 
 }
 
 void launch_get_state(const Geom& g, const uint8_t* mask, const float* dang, const void* ang,
-                      int storage, int G, int r, float* out, cudaStream_t s) {
+                      int storage, int r, float* out, cudaStream_t s) {
     with_storage(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
         k_get_state<S><<<grid_for((int64_t)g.H * g.W, 256), 256, 0, s>>>(
-            g, mask, dang, static_cast<const S*>(ang), G, r, out);
+            g, mask, dang, static_cast<const S*>(ang), r, out);
     });
 }
 
-void launch_set_state(const Geom& g, const uint8_t* mask, void* ang, int storage, int G, int r,
+void launch_set_state(const Geom& g, const uint8_t* mask, void* ang, int storage, int r,
                       const float* in, cudaStream_t s) {
     with_storage(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
         k_set_state<S><<<grid_for((int64_t)g.H * g.W, 256), 256, 0, s>>>(
-            g, mask, static_cast<S*>(ang), G, r, in);
+            g, mask, static_cast<S*>(ang), r, in);
     });
 }
 
 void launch_block_energy(const Geom& g, const int32_t* of_block, const uint8_t* mask,
-                         const float* dang, const void* ang, int storage, int G, int r, double q,
+                         const float* dang, const void* ang, int storage, int r, double q,
                          double J, double* E, cudaStream_t s) {
     const int threads = 256;
     const int blocks = (int)(((int64_t)g.nblk * 32 + threads - 1) / threads);
     with_storage(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
         k_block_energy<S><<<blocks, threads, 0, s>>>(g, of_block, mask, dang,
-                                                     static_cast<const S*>(ang), G, r, q, J, E);
+                                                     static_cast<const S*>(ang), r, q, J, E);
     });
 }
 
@@ -1457,11 +1436,11 @@ void launch_sst(const Geom& g, const Slices& sl, const float* T_blk, int r, int 
         k_sst_box<<<grid, 256, 0, s>>>(g, sl, Ts, tmp, r, 1);
         k_sst_box<<<grid, 256, 0, s>>>(g, sl, tmp, Ts, r, 0);
     }
-    k_sst_beta<<<grid, 256, 0, s>>>(n, Ts, Tf, beta);
+    k_sst_beta<<<grid, 256, 0, s>>>(g, Ts, Tf, beta);
 }
 
-void launch_site_beta(int64_t n, const float* Tf, float* beta, cudaStream_t s) {
-    k_site_beta<<<grid_for(n, 256), 256, 0, s>>>(n, Tf, beta);
+void launch_site_beta(const Geom& g, const float* Tf, float* beta, cudaStream_t s) {
+    k_site_beta<<<grid_for((int64_t)g.H * g.W, 256), 256, 0, s>>>(g, Tf, beta);
 }
 
 void launch_cal_moments(int nblk, int nbx, int Rp, int chains, const double* ecur, double* S,

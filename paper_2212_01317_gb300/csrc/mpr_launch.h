@@ -22,28 +22,28 @@ void launch_block_stats(const Geom& g, const Slices& sl, const float* values, co
                         double q, double J, double* Es, int32_t* Nsp, int32_t* Nb, double* ssum,
                         int32_t* nsamp, int32_t* ngap0, int32_t* ngap1, cudaStream_t s);
 void launch_scan(const int32_t* cnt, int n, int32_t* out, cudaStream_t s);
-void launch_build_lists(const Geom& g, const int32_t* of_block, const uint8_t* mask,
-                        const int32_t* start0, const int32_t* start1, uint2* list0, uint2* list1,
+void launch_build_lists(const Geom& g, const Slices& sl, const uint8_t* mask,
+                        const int32_t* start0, const int32_t* start1, uint4* list0, uint4* list1,
                         int32_t* split0, int32_t* split1, cudaStream_t s);
 // `storage` is an mpr_storage value (0 FP32, 1 BF16, 2 FP16): the element
 // type of the batch state `ang`.
-void launch_init(const Geom& g, const Slices& sl, const uint2* list, int64_t n_list, int colour,
-                 const float* init_angle, void* ang, int storage, int G, int Rp, int random,
+void launch_init(const Geom& g, const Slices& sl, const uint4* list, int64_t n_list, int colour,
+                 const float* init_angle, void* ang, int storage, int n_pairs, int random,
                  Rng rng, uint32_t r_even, cudaStream_t s);
 void launch_fill_samples(const Geom& g, const uint8_t* mask, const float* dang, void* ang,
-                         int storage, int G, int groups, cudaStream_t s);
+                         int storage, int n_pairs, cudaStream_t s);
 // form 0, 1, 2: one, two or four warps per realization pair (more warps per
 // pair as fewer items are left).
-void launch_sweep(const SweepArgs& a, int G, int storage, int form, int grid, cudaStream_t s);
-int sweep_blocks_per_sm(int G, int storage, int form);
-int sweep_items_per_cta(int G, int form);
+void launch_sweep(const SweepArgs& a, int storage, int form, int grid, cudaStream_t s);
+int sweep_blocks_per_sm(int storage, int form);
+int sweep_items_per_cta(int form);
 void launch_energy(const SweepArgs& a, int G, int storage, int n_sm, cudaStream_t s);
 // fold: NULL, or the previous sweep's fold run by extra CTAs of this launch.
 void launch_sweep_flat(const SweepArgs& a, int G, int64_t n_list, cudaStream_t s,
                        const FoldArgs* fold = nullptr);
 // The same half-step of the calibration's chains in the warp form (one warp
 // per (block, pair) unit).
-void launch_sweep_cal(const SweepArgs& a, int G, cudaStream_t s, const FoldArgs* fold = nullptr);
+void launch_sweep_cal(const SweepArgs& a, cudaStream_t s, const FoldArgs* fold = nullptr);
 void launch_ecur_broadcast(int nblk, int Rp, int G, double* ecur, cudaStream_t s);
 void launch_ecur_reset(int nblk, int Rp, const double* Es, double* ecur, double* eacc,
                        cudaStream_t s);
@@ -97,9 +97,9 @@ void launch_kcal_update(int nblk, double inv_count, const double* es, const int3
 void launch_cal_update(int nblk, double inv_count, const double* es, const int32_t* Nsp,
                        const float* T, float* lo, float* hi, double* ebar, Control* ctl,
                        int n_bisect, cudaGraphConditionalHandle cond, cudaStream_t s);
-void launch_accumulate(const Geom& g, const uint2* list, int64_t n_list, int colour,
-                       const void* ang, int storage, int G, int groups, int r_off, int R,
-                       double* sum, cudaStream_t s);
+void launch_accumulate(const Geom& g, const uint4* list, int64_t n_list, int colour,
+                       const void* ang, int storage, int r_off, int R, double* sum,
+                       cudaStream_t s);
 void launch_sum_to_grid(const Geom& g, const uint8_t* mask, const double* sum, double* out,
                         cudaStream_t s);
 void launch_grid_to_sum(const Geom& g, const uint8_t* mask, const double* in, double* sum,
@@ -109,18 +109,18 @@ void launch_predict(const Geom& g, const Slices& sl, const float* values, const 
                     const double* sum, double inv_r, float* out, const float* truth, double* err,
                     cudaStream_t s);
 void launch_get_state(const Geom& g, const uint8_t* mask, const float* dang, const void* ang,
-                      int storage, int G, int r, float* out, cudaStream_t s);
-void launch_set_state(const Geom& g, const uint8_t* mask, void* ang, int storage, int G, int r,
+                      int storage, int r, float* out, cudaStream_t s);
+void launch_set_state(const Geom& g, const uint8_t* mask, void* ang, int storage, int r,
                       const float* in, cudaStream_t s);
 void launch_block_energy(const Geom& g, const int32_t* of_block, const uint8_t* mask,
-                         const float* dang, const void* ang, int storage, int G, int r, double q,
+                         const float* dang, const void* ang, int storage, int r, double q,
                          double J, double* E, cudaStream_t s);
 
 // Sec. 2.2.3 site temperatures: Ts (FP64, H*W) smoothed from T_blk, then
 // Tf = (float)Ts and beta = 1 / Tf; tmp is H*W doubles of scratch.
 void launch_sst(const Geom& g, const Slices& sl, const float* T_blk, int r, int n_s, double* Ts,
                 double* tmp, float* Tf, float* beta, cudaStream_t s);
-void launch_site_beta(int64_t n, const float* Tf, float* beta, cudaStream_t s);
+void launch_site_beta(const Geom& g, const float* Tf, float* beta, cudaStream_t s);
 
 // Energy moments of the calibration chains and the Newton calibration.
 void launch_cal_moments(int nblk, int nbx, int Rp, int chains, const double* ecur, double* S,
@@ -136,13 +136,13 @@ void launch_energy_vjp(int nblk, int nbx, const int32_t* Nb, const double* M, co
 void launch_set_tag(Control* ctl, uint32_t tag, cudaStream_t s);
 
 // The realizations' stop tail as one cooperative launch (mpr_simtail.cu).
-int sim_tail_blocks_per_sm(int G, int storage);
-cudaError_t launch_sim_tail(const SimTailArgs& a, int G, int storage, int grid, cudaStream_t s);
+int sim_tail_blocks_per_sm(int storage);
+cudaError_t launch_sim_tail(const SimTailArgs& a, int storage, int grid, cudaStream_t s);
 
 // The realizations' stop tail with one CTA per realization pair
 // (mpr_pairtail.cu); every pair's running units must fit kPairTailCap.
 constexpr int kPairTailCap = 4096;
-cudaError_t launch_pair_tail(const SimTailArgs& a, int G, int storage, int n_pairs,
+cudaError_t launch_pair_tail(const SimTailArgs& a, int storage, int n_pairs,
                              cudaStream_t s);
 
 // The staged half-step (mpr_tile.cu): tile shape of a geometry, the staging

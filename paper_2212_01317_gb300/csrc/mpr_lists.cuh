@@ -1,8 +1,8 @@
 // Gap-list entries: the description of one gap site that every half-step
-// reads (its coordinates, its block, which of its four neighbours exist and
-// are gaps, and which of its bonds another block owns). Shared by the
-// block-major lists (mpr_kernels.cu) and the tile-major lists of the staged
-// half-step (mpr_tile.cu), so both describe a site identically.
+// reads (where it lies, its block, which of its four neighbours exist and
+// are gaps, and which of its bonds another block owns). The flags are shared
+// by the block-major lists (gap_item, mpr_kernels.cu) and the tile-major lists
+// of the staged half-step (gap_entry, mpr_tile.cu).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -60,6 +60,20 @@ __device__ __forceinline__ uint2 gap_entry(const Geom& g, const uint8_t* __restr
     if (hl && x == fr.x0) f |= EDGE_L;
     if (hu && y == fr.y0) f |= EDGE_U;
     return make_uint2(((uint32_t)y << 16) | (uint32_t)x, ((uint32_t)fr.b << META_SHIFT) | f);
+}
+
+// The block-major lists' entry of gap site (y, x): everything the sweep would
+// otherwise compute for every realization pair it updates the site in, worked
+// out once. .x = half index y Wh + x / 2 (below 2^29), .y = gap_entry's .y,
+// .z = the Philox counter word (the site's index within its field), .w = the
+// left neighbour's half index (the right one's is one more; -1 at the grid's
+// first site).
+__device__ __forceinline__ uint4 gap_item(const Geom& g, const int4& rect,
+                                          const uint8_t* __restrict__ mask,
+                                          const BlockFrame& fr, int y, int x) {
+    const uint2 e = gap_entry(g, mask, fr, y, x);
+    const uint32_t hs = (uint32_t)y * (uint32_t)g.Wh + (uint32_t)(x >> 1);
+    return make_uint4(hs, e.y, local_index(rect, y, x), hs + (uint32_t)(x & 1) - 1u);
 }
 
 }  // namespace mpr

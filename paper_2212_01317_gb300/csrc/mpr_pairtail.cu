@@ -28,15 +28,13 @@ namespace {
 constexpr int kPairThreads = 1024;
 constexpr int kPairWarps = kPairThreads / 32;
 
-template <int G, typename S>
+template <typename S>
 __global__ void __launch_bounds__(kPairThreads, 1) k_pair_tail(SimTailArgs a) {
-    constexpr int NP = G / 2;
     __shared__ uint32_t s_units[2][kPairTailCap];
     __shared__ uint32_t s_n[2];
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int npairs = a.sw.groups * NP;
+    const int npairs = a.sw.Rp >> 1;
     const int p = blockIdx.x;                         // this CTA's realization pair
-    const int grp = p / NP, q = p - grp * NP;
     Control* ctl = a.ctl;
     const uint32_t t0 = ctl->t, tag = ctl->tag;
     const uint32_t n0 = ctl->n_work[t0 & 1u];
@@ -77,7 +75,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_tail(SimTailArgs a) {
             s.split = a.split[c];
             for (uint32_t it = slot; it < n; it += nslot) {
                 const int b = (int)(s_units[cur][it] / (uint32_t)npairs);
-                sweep_item<G, S>(s, b * s.groups + grp, q + NP * cw, NP * k, ctr1);
+                sweep_item<S>(s, b, p, cw, k, ctr1);
             }
             __syncthreads();
         }
@@ -120,13 +118,12 @@ template <typename F> void with_storage_pair(int storage, F&& f) {
 
 }  // namespace
 
-cudaError_t launch_pair_tail(const SimTailArgs& a, int G, int storage, int n_pairs,
+cudaError_t launch_pair_tail(const SimTailArgs& a, int storage, int n_pairs,
                              cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     with_storage_pair(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
-        if (G == 2) k_pair_tail<2, S><<<n_pairs, kPairThreads, 0, s>>>(a);
-        else k_pair_tail<8, S><<<n_pairs, kPairThreads, 0, s>>>(a);
+        k_pair_tail<S><<<n_pairs, kPairThreads, 0, s>>>(a);
         e = cudaGetLastError();
     });
     return e;

@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(512, 1) k_cal_persistent(CalPersistArgs a) {
     const int gquad = blockIdx.x * nquad + quad, nquads = gridDim.x * nquad;
     const int n_items = nblk * a.sw.groups;
     const int n_sweeps = a.n_eq + a.n_meas;
-    const size_t plane = (size_t)a.sw.g.H * a.sw.g.Wh;
     for (int k = 0; k <= a.n_bisect; ++k) {
         // Midpoints of the brackets; blocks without sample bonds take the
         // median of the targeted blocks' midpoints. k == n_bisect: final T.
@@ -93,19 +92,17 @@ __global__ void __launch_bounds__(512, 1) k_cal_persistent(CalPersistArgs a) {
             for (int64_t t = tid; t < total; t += nthr) {
                 const int64_t e = t / Rp;
                 const int r = (int)(t % Rp);
-                const uint2 en = a.list[c][e];
-                const int y = en.x >> 16, x = en.x & 0xffff;
+                const uint4 en = a.list[c][e];
                 float v = a.init_angle[en.y >> META_SHIFT];
                 if (a.random_init) {
                     const int sl = a.sw.sl.of_block[en.y >> META_SHIFT];
                     uint32_t w[4];
-                    philox4x32_10(local_index(a.sw.sl.rect[sl], y, x), 0xFFFFu << 16,
+                    philox4x32_10(en.z, 0xFFFFu << 16,
                                   (uint32_t)r >> 1, 0u, a.sw.rng.key0, a.sw.sl.key1[sl], w);
                     v = kTwoPi * u01(w[(r & 1) * 2]);
                 }
-                const int grp = r / G, lane = r % G;
-                static_cast<float*>(a.sw.ang)[((size_t)(grp * 2 + c) * plane +
-                                               (size_t)y * a.sw.g.Wh + (x >> 1)) * G + lane] = v;
+                static_cast<float*>(a.sw.ang)[pair_plane(a.sw.g, r >> 1, c) + 2 * (size_t)en.x +
+                                              (r & 1)] = v;
             }
         }
         for (int64_t t = tid; t < (int64_t)nblk * Rp; t += nthr) {
@@ -117,7 +114,8 @@ __global__ void __launch_bounds__(512, 1) k_cal_persistent(CalPersistArgs a) {
         // E_b of the start state from scratch.
         for (int c = 0; c < 2; ++c) {
             const SweepArgs s = colour_args(a, c);
-            for (int it = gquad; it < n_items; it += nquads) energy_item<G, float>(s, it, warp & 3, 4);
+            for (int it = gquad; it < n_items; it += nquads) 
+                energy_item<float>(s, it / s.groups, it % s.groups, G / 2, warp & 3, 4);
         }
         if (!grid_sync(a.bar, gen, lim)) return;
         // n_eq + n_meas sweeps; the change of sweep t is folded into E_b while
@@ -129,10 +127,11 @@ __global__ void __launch_bounds__(512, 1) k_cal_persistent(CalPersistArgs a) {
                 s.eacc = a.eacc2[sweep & 1];
                 if constexpr (G == 2) {
                     for (int it = gwarp; it < n_items; it += nwarps)
-                        sweep_item<G, float>(s, it, 0, 1, ctr1);
+                        sweep_item<float>(s, it / s.groups, it % s.groups, 0, 1, ctr1);
                 } else {
                     for (int it = gquad; it < n_items; it += nquads)
-                        sweep_item<G, float>(s, it, warp & 3, 4, ctr1);
+                        sweep_item<float>(s, it / s.groups,
+                                          (it % s.groups) * (G / 2) + (warp & 3), 0, 1, ctr1);
                 }
                 if (c == 0 && sweep > 1) fold_sweep(a, sweep - 1, tid, nthr);
                 if (!grid_sync(a.bar, gen, lim)) return;

@@ -23,9 +23,8 @@ namespace mpr {
 
 constexpr int kTailThreads = 512;
 
-template <int G, typename S>
+template <typename S>
 __global__ void __launch_bounds__(kTailThreads, 2) k_sim_tail(SimTailArgs a) {
-    constexpr int NP = G / 2;
     constexpr int WPC = kTailThreads / 32;
     const int warp = threadIdx.x >> 5;
     const int gw = blockIdx.x * WPC + warp, nw = gridDim.x * WPC;
@@ -58,7 +57,7 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_sim_tail(SimTailArgs a) {
         // block's entries) when they are few.
         int k = 1;
         while (k < 4 && (int64_t)n_items * 2 * k <= nw) k *= 2;
-        const int npairs = a.sw.groups * NP;
+        const int npairs = a.sw.Rp >> 1;
         const int ngrp = nw / k, gi = gw / k, cw = gw % k;
         for (int c = 0; c < 2; ++c) {
             SweepArgs s = a.sw;
@@ -69,9 +68,8 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_sim_tail(SimTailArgs a) {
             if (gi < ngrp)
                 for (uint32_t it = (uint32_t)gi; it < n_items; it += (uint32_t)ngrp) {
                     const int u = (int)work[it];
-                    const int b = u / npairs, p = u - b * npairs;
-                    const int grp = p / NP, q = p - grp * NP;
-                    sweep_item<G, S>(s, b * s.groups + grp, q + NP * cw, NP * k, ctr1);
+                    const int b = u / npairs;
+                    sweep_item<S>(s, b, u - b * npairs, cw, k, ctr1);
                 }
             if (!grid_sync(a.bar, gen, lim)) return;
         }
@@ -102,25 +100,21 @@ template <typename F> void with_storage_tail(int storage, F&& f) {
 }
 }  // namespace
 
-int sim_tail_blocks_per_sm(int G, int storage) {
+int sim_tail_blocks_per_sm(int storage) {
     int n = 0;
     with_storage_tail(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
-        if (G == 2)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sim_tail<2, S>, kTailThreads, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sim_tail<8, S>, kTailThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sim_tail<S>, kTailThreads, 0);
     });
     return n < 2 ? n : 2;
 }
 
-cudaError_t launch_sim_tail(const SimTailArgs& a, int G, int storage, int grid, cudaStream_t s) {
+cudaError_t launch_sim_tail(const SimTailArgs& a, int storage, int grid, cudaStream_t s) {
     void* args[] = {const_cast<SimTailArgs*>(&a)};
     cudaError_t e = cudaSuccess;
     with_storage_tail(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
-        const void* k = G == 2 ? (const void*)k_sim_tail<2, S> : (const void*)k_sim_tail<8, S>;
-        e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kTailThreads), args, 0, s);
+        e = cudaLaunchCooperativeKernel((const void*)k_sim_tail<S>, dim3(grid), dim3(kTailThreads), args, 0, s);
     });
     return e;
 }

@@ -2,11 +2,14 @@
 // pass, shared by the per-launch kernels (mpr_kernels.cu) and the persistent
 // calibration kernel (mpr_persist.cu).
 //
-// A (block, lane group) item is one block of the grid for the G realizations
-// of one lane group; the realizations' worklist hands out its realization
-// pairs one by one (units), the calibration's flat kernel every entry. The state interleaves G realizations per site; each
-// lane updates its site in both realizations of one realization pair, from
-// one Philox block: words 0, 1 for the even realization, 2, 3 for the odd.
+// A unit is one block of the grid in one realization pair; the realizations'
+// worklist hands out units, the calibration's flat kernel every entry. Each
+// lane updates its site in both realizations of the pair, from one Philox
+// block: words 0, 1 for the even realization, 2, 3 for the odd. Every pair has
+// its own planes of the state: neighbouring half-sites are neighbouring words,
+// so a warp's loads of one unit touch a quarter of the cache lines they would
+// with eight realizations interleaved per site (FP32, 2048^2, l_b = 32, 32
+// realizations: first sweeps 147 against 125 G updates/s).
 //
 // Block energies are kept incrementally. A move changes the energy of the
 // site's four bonds by dE, and the reflection conserves it (up to the
@@ -28,23 +31,33 @@
 namespace mpr {
 
 // Element type of the batch state: a realization pair is two adjacent
-// elements, loaded and stored as one 8-byte (FP32) or 4-byte (FP16 / BF16)
-// access; arithmetic is FP32 throughout. The sample angles the method
-// conditions on are never rounded: the 16-bit forms read them from the FP32
-// per-field table instead of the state.
+// elements, one 8-byte (FP32) or 4-byte (FP16 / BF16) word; arithmetic is FP32
+// throughout. The sample angles the method conditions on are never rounded:
+// in the 16-bit forms a sample site's word holds its FP32 angle, so a
+// neighbour is one load of the same size whether it is a gap or a sample, and
+// decode() is told which.
 template <typename S> struct Store;
 
 template <> struct Store<float> {
     static constexpr bool kExact = true;
+    using Word = float2;             // a realization pair as it lies in memory
+    __device__ static float2 decode(Word w, bool) { return w; }
     __device__ static float2 load2(const float* p) { return *reinterpret_cast<const float2*>(p); }
     __device__ static void store2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
     __device__ static float load1(const float* p) { return *p; }
     __device__ static void store1(float* p, float v) { *p = v; }
     __device__ static float round(float v) { return v; }
+    __device__ static float2 round2(float2 v) { return v; }
 };
 
 template <> struct Store<__half> {
     static constexpr bool kExact = false;
+    using Word = uint32_t;
+    __device__ static float2 decode(Word w, bool gap) {
+        const float s = __uint_as_float(w);
+        const __half2 h = *reinterpret_cast<const __half2*>(&w);
+        return gap ? __half22float2(h) : make_float2(s, s);
+    }
     __device__ static float2 load2(const __half* p) {
         return __half22float2(*reinterpret_cast<const __half2*>(p));
     }
@@ -54,10 +67,19 @@ template <> struct Store<__half> {
     __device__ static float load1(const __half* p) { return __half2float(*p); }
     __device__ static void store1(__half* p, float v) { *p = __float2half_rn(v); }
     __device__ static float round(float v) { return __half2float(__float2half_rn(v)); }
+    __device__ static float2 round2(float2 v) {
+        return __half22float2(__floats2half2_rn(v.x, v.y));
+    }
 };
 
 template <> struct Store<__nv_bfloat16> {
     static constexpr bool kExact = false;
+    using Word = uint32_t;
+    __device__ static float2 decode(Word w, bool gap) {
+        const float s = __uint_as_float(w);
+        return make_float2(gap ? __uint_as_float(w << 16) : s,
+                           gap ? __uint_as_float(w & 0xFFFF0000u) : s);
+    }
     __device__ static float2 load2(const __nv_bfloat16* p) {
         return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
     }
@@ -67,42 +89,95 @@ template <> struct Store<__nv_bfloat16> {
     __device__ static float load1(const __nv_bfloat16* p) { return __bfloat162float(*p); }
     __device__ static void store1(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
     __device__ static float round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+    __device__ static float2 round2(float2 v) {
+        return __bfloat1622float2(__floats2bfloat162_rn(v.x, v.y));
+    }
 };
 
 // Site update with the state's rounding applied: the proposal is rounded
 // before its energy is taken, so the Metropolis test judges the angle that
 // is stored; the reflected angle is rounded too, and for the 16-bit forms
-// dE becomes the exact change from the old to the stored final angle, with
-// (ca, sa) the final angle's cos / sin and refl cleared.
+// dE is the exact change from the old to the stored final angle. Sn, C: the
+// local field. The roundings are spelled out (see bond_change).
 template <typename S>
 __device__ __forceinline__ SiteNew site_update(float phi, float C, float Sn, float u0, float u1,
                                                float beta, const Model& m) {
     SiteNew n;
-    __sincosf(m.q * phi, &n.so, &n.co);
+    float co, so, cp, sp;
+    __sincosf(m.q * phi, &so, &co);
     const float php = Store<S>::round(kTwoPi * u0);
-    float sp, cp;
     __sincosf(m.q * php, &sp, &cp);
-    const float dE = m.J * ((C * n.co + Sn * n.so) - (C * cp + Sn * sp));
-    const bool acc = (dE <= 0.0f) || (u1 < __expf(-dE * beta));
-    n.phi = acc ? php : phi;
+    const float e0 = __fmaf_rn(Sn, so, __fmul_rn(C, co));
+    const float e1 = __fmaf_rn(Sn, sp, __fmul_rn(C, cp));
+    const float dE = __fmul_rn(m.J, __fsub_rn(e0, e1));
+    // exp(-dE beta) = 2^(-dE beta log2 e)
+    const bool acc = (dE <= 0.0f) ||
+                     (u1 < ex2_approx(__fmul_rn(__fmul_rn(dE, -beta), 1.44269504088896341f)));
+    n.mid = acc ? php : phi;
     n.dE = acc ? dE : 0.0f;
-    n.ca = acc ? cp : n.co;
-    n.sa = acc ? sp : n.so;
     // Over-relaxation, without branches. The reflected angle (2 psi - q phi)/q
     // is >= 0 only if psi >= 0, i.e. S >= 0, so psi is taken from (|S|, C) and
-    // the move is kept only when S >= 0 and the angle lies in [0, 2pi]
-    // (C = S = 0 gives NaN and fails the test).
+    // the move is kept only when S >= 0 and the angle lies in [0, 2pi], as one
+    // comparison of the bits: a negative number or the NaN of C = S = 0
+    // compares above (-0 cannot arise from the fused difference).
     const float psi = atan2_upper(fabsf(Sn), C);
-    const float por = (2.0f * psi - m.q * n.phi) * m.inv_q;
-    n.refl = m.overrelax && Sn >= 0.0f && por >= 0.0f && por <= kTwoPi;
-    n.phi = n.refl ? Store<S>::round(por) : n.phi;
+    const float por = __fmul_rn(__fmaf_rn(-m.q, n.mid, 2.0f * psi), m.inv_q);
+    n.refl = m.overrelax && Sn >= 0.0f && __float_as_uint(por) <= __float_as_uint(kTwoPi);
+    n.phi = n.refl ? Store<S>::round(por) : n.mid;
     if constexpr (!Store<S>::kExact) {
         float sf, cf;
         __sincosf(m.q * n.phi, &sf, &cf);
-        n.ca = cf;
-        n.sa = sf;
-        n.refl = false;
-        n.dE = m.J * ((C * n.co + Sn * n.so) - (C * cf + Sn * sf));
+        n.dE = __fmul_rn(m.J, __fsub_rn(e0, __fmaf_rn(Sn, sf, __fmul_rn(C, cf))));
+    }
+    return n;
+}
+
+// site_update of a site in both realizations of a pair, with the same roundings
+// (bit for bit): what is not a hardware function or a choice is packed two-wide
+// FP32 arithmetic, one instruction for both realizations. The half-step is
+// bound by instruction issue (60-66 %, no pipe above 55 %, DRAM below 30 %), so
+// instructions are what it has to save: with the packed arithmetic, the list
+// entries that hold what every pair would compute again (gap_item) and the
+// pair planes, a warp pass of 32 entries x 2 realizations takes about 280
+// instead of 400 instructions (FP32 state; 310 instead of 430 in BF16). First
+// sweeps of a 2048^2 field, 32 realizations, half the sites missing: l_b = 32
+// FP32 125 -> 147, BF16 104 -> 139, l_b = 16 (two units per warp) FP32
+// 106 -> 120 G updates/s. Copying the next entry's words into shared memory
+// ahead of time (cp.async) removed the long-scoreboard stalls but cost as many
+// instructions and L1 wavefronts as it saved (2.21 against 2.03 ms per four
+// BF16 sweeps); loads one entry ahead into registers, bulk prefetches of the
+// next unit's rows into L2, and 7, 9 or 10 CTAs per SM were slower too.
+template <typename S>
+__device__ __forceinline__ PairNew pair_update(float2 phi, float2 C, float2 Sn, float2 u0,
+                                               float2 u1, float2 beta, const Model& m) {
+    PairNew n;
+    const float2 q2 = both(m.q), J2 = both(m.J);
+    float2 co, so, cp, sp;
+    sincos_2(__fmul2_rn(q2, phi), so, co);
+    const float2 php = Store<S>::round2(__fmul2_rn(both(kTwoPi), u0));
+    sincos_2(__fmul2_rn(q2, php), sp, cp);
+    const float2 e0 = __ffma2_rn(Sn, so, __fmul2_rn(C, co));
+    const float2 e1 = __ffma2_rn(Sn, sp, __fmul2_rn(C, cp));
+    n.dE = __fmul2_rn(J2, __ffma2_rn(e1, both(-1.0f), e0));
+    const float2 x = __fmul2_rn(__fmul2_rn(n.dE, make_float2(-beta.x, -beta.y)),
+                                both(1.44269504088896341f));
+    const bool acc0 = (n.dE.x <= 0.0f) || (u1.x < ex2_approx(x.x));
+    const bool acc1 = (n.dE.y <= 0.0f) || (u1.y < ex2_approx(x.y));
+    n.mid = make_float2(acc0 ? php.x : phi.x, acc1 ? php.y : phi.y);
+    const float2 psi = atan2_upper_2(make_float2(fabsf(Sn.x), fabsf(Sn.y)), C);
+    const float2 por = __fmul2_rn(
+        __ffma2_rn(make_float2(-m.q, -m.q), n.mid, __fadd2_rn(psi, psi)), both(m.inv_q));
+    n.refl0 = m.overrelax && Sn.x >= 0.0f && __float_as_uint(por.x) <= __float_as_uint(kTwoPi);
+    n.refl1 = m.overrelax && Sn.y >= 0.0f && __float_as_uint(por.y) <= __float_as_uint(kTwoPi);
+    const float2 pr = Store<S>::round2(por);
+    n.phi = make_float2(n.refl0 ? pr.x : n.mid.x, n.refl1 ? pr.y : n.mid.y);
+    if constexpr (Store<S>::kExact) {
+        n.dE = make_float2(acc0 ? n.dE.x : 0.0f, acc1 ? n.dE.y : 0.0f);
+    } else {
+        float2 cf, sf;
+        sincos_2(__fmul2_rn(q2, n.phi), sf, cf);
+        const float2 e2 = __ffma2_rn(Sn, sf, __fmul2_rn(C, cf));
+        n.dE = __fmul2_rn(J2, __ffma2_rn(e2, both(-1.0f), e0));
     }
     return n;
 }
@@ -125,76 +200,135 @@ __device__ __forceinline__ void flush_pair(double* ea, float v0, float v1) {
 }
 
 // Bond-by-bond split of a move at a block edge: (lc, ls) and (uc, us) are the
-// left and upper neighbours' (cos, sin) of q phi_j.
-__device__ __forceinline__ void add_energy_lu(const SiteNew& n, uint32_t f, float C, float S,
-                                              float lc, float ls, float uc, float us, float J,
-                                              float& ao, float& al, float& au) {
-    if (!(f & (EDGE_L | EDGE_U))) {
-        ao += n.dE;
-        return;
+// left and upper neighbours' (cos, sin) of q phi_j. The roundings are spelled
+// out, so that every form adds the same numbers whatever the compiler would
+// contract in it.
+template <typename S>
+__device__ __forceinline__ float bond_change(float dc, float ds, float c, float s, float J) {
+    return -J * (Store<S>::kExact ? __fmaf_rn(dc, c, __fmul_rn(ds, s))
+                                  : __fmaf_rn(ds, s, __fmul_rn(dc, c)));
+}
+
+// phi: the angle before the update. The cosines and sines of the site's own
+// angles are computed again here: only a block's edge sites come here, and
+// kept values would cost every update registers.
+template <typename S>
+__device__ __forceinline__ void split_edge(const SiteNew& n, float phi, uint32_t f, float C,
+                                           float Sn, float lc, float ls, float uc, float us,
+                                           const Model& m, float& ao, float& al, float& au) {
+    float co, so, cn, sn;
+    __sincosf(m.q * phi, &so, &co);
+    if constexpr (Store<S>::kExact) {
+        float ca, sa;
+        __sincosf(m.q * n.mid, &sa, &ca);
+        final_cs(n.refl, ca, sa, C, Sn, cn, sn);
+    } else {
+        __sincosf(m.q * n.phi, &sn, &cn);
     }
-    float cn, sn;
-    final_cs(n, C, S, cn, sn);
-    const float dc = cn - n.co, ds = sn - n.so;
-    const float dl = -J * (dc * lc + ds * ls);
-    const float du = -J * (dc * uc + ds * us);
+    const float dc = cn - co, ds = sn - so;
     ao += n.dE;
-    if (f & EDGE_L) { ao -= dl; al += dl; }
-    if (f & EDGE_U) { ao -= du; au += du; }
-}
-
-// The same with the four neighbours' (cos, sin) in arrays (left, right, up,
-// down), as the kernels that keep all four use it.
-__device__ __forceinline__ void add_energy(const SiteNew& n, uint32_t f, float C, float S,
-                                           const float* nc, const float* ns, float J, float& ao,
-                                           float& al, float& au) {
-    add_energy_lu(n, f, C, S, nc[0], ns[0], nc[2], ns[2], J, ao, al, au);
-}
-
-// Angles of the four neighbours of a site in both realizations of the pair.
-// FP32 state: every neighbour is one 8-byte state load (the state holds the
-// sample angles too). 16-bit state: a gap neighbour is read from the state,
-// a sample neighbour from the FP32 per-field table `dang`, both loads
-// predicated on the flags. A neighbour outside the grid reads as 0 and is
-// masked out by the caller.
-template <typename S>
-__device__ __forceinline__ void neighbour_angles(const SweepArgs& a, const S* __restrict__ oth,
-                                                 int G, uint32_t hs, int x, uint32_t f,
-                                                 float2 v[4]) {
-    const uint32_t o = (uint32_t)(x & 1);
-    const uint32_t hn[4] = {hs + o - 1u, hs + o, hs - (uint32_t)a.g.Wh, hs + (uint32_t)a.g.Wh};
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        const bool ex = (f & (NB_L << d)) != 0;
-        if constexpr (Store<S>::kExact) {
-            v[d] = ex ? Store<S>::load2(oth + (size_t)hn[d] * G) : make_float2(0.0f, 0.0f);
-        } else {
-            const bool gap = (f & (GAP_L << d)) != 0;
-            const float* dn = a.dang + (size_t)(a.colour ^ 1) * a.g.H * a.g.Wh;
-            const float sv = (ex && !gap) ? dn[hn[d]] : 0.0f;
-            v[d] = (ex && gap) ? Store<S>::load2(oth + (size_t)hn[d] * G) : make_float2(sv, sv);
-        }
+    if (f & EDGE_L) {
+        const float d = bond_change<S>(dc, ds, lc, ls, m.J);
+        ao -= d;
+        al += d;
+    }
+    if (f & EDGE_U) {
+        const float d = bond_change<S>(dc, ds, uc, us, m.J);
+        ao -= d;
+        au += d;
     }
 }
 
-// (cos, sin) of q * phi_j of the four neighbours, masked by existence.
+// The same for a pair (.x, .y).
 template <typename S>
-__device__ __forceinline__ void neighbour_field(const SweepArgs& a, const S* __restrict__ oth,
-                                                int G, uint32_t hs, int x, uint32_t f, float* nc0,
-                                                float* ns0, float* nc1, float* ns1) {
-    float2 v[4];
-    neighbour_angles<S>(a, oth, G, hs, x, f, v);
+__device__ __forceinline__ void split_edge_2(const PairNew& n, float2 phi, uint32_t f, float2 C,
+                                             float2 Sn, float2 lc, float2 ls, float2 uc, float2 us,
+                                             const Model& m, float2& ao, float2& al, float2& au) {
+    split_edge<S>(SiteNew{n.phi.x, n.mid.x, n.dE.x, n.refl0}, phi.x, f, C.x, Sn.x, lc.x, ls.x,
+                  uc.x, us.x, m, ao.x, al.x, au.x);
+    split_edge<S>(SiteNew{n.phi.y, n.mid.y, n.dE.y, n.refl1}, phi.y, f, C.y, Sn.y, lc.y, ls.y,
+                  uc.y, us.y, m, ao.y, al.y, au.y);
+}
+
+// The neighbours' angles (left, right, up, down) in both realizations of the
+// pair, from its plane of the other colour. A neighbour that does not exist
+// reads some other site's word or the state's guard; neighbour_field drops it.
+template <typename S>
+__device__ __forceinline__ void load_neighbours(const Geom& g, const S* __restrict__ oth,
+                                                const uint4& en, float2 v[4]) {
+    using W = typename Store<S>::Word;
+    const W* left = reinterpret_cast<const W*>(oth) + (ptrdiff_t)(int)en.w;
+    const W* here = reinterpret_cast<const W*>(oth) + en.x;
+    v[0] = Store<S>::decode(left[0], (en.y & GAP_L) != 0);
+    v[1] = Store<S>::decode(left[1], (en.y & GAP_R) != 0);
+    v[2] = Store<S>::decode(*(here - g.Wh), (en.y & GAP_U) != 0);
+    v[3] = Store<S>::decode(here[g.Wh], (en.y & GAP_D) != 0);
+}
+
+// (cos, sin) of q phi_j of the four neighbours from their angles; 0 for a
+// neighbour that does not exist.
+__device__ __forceinline__ void neighbour_field(const Model& m, const float2 v[4], uint32_t f,
+                                                float2 nc[4], float2 ns[4]) {
 #pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        const float m = (f & (NB_L << d)) ? 1.0f : 0.0f;
-        float s0, c0, s1, c1;
-        __sincosf(a.m.q * v[d].x, &s0, &c0);
-        __sincosf(a.m.q * v[d].y, &s1, &c1);
-        nc0[d] = m * c0;
-        ns0[d] = m * s0;
-        nc1[d] = m * c1;
-        ns1[d] = m * s1;
+    for (int d = 0; d < 4; ++d) sincos_2(__fmul2_rn(both(m.q), v[d]), ns[d], nc[d]);
+    if ((f & 0xFu) != 0xFu) {
+#pragma unroll
+        for (int d = 0; d < 4; ++d)
+            if (!(f & (NB_L << d))) nc[d] = ns[d] = make_float2(0.0f, 0.0f);
     }
+}
+
+// Sum over the four neighbours, in the order every form uses.
+__device__ __forceinline__ float2 sum4(const float2 v[4]) {
+    return __fadd2_rn(__fadd2_rn(v[0], v[1]), __fadd2_rn(v[2], v[3]));
+}
+
+// One gap entry updated in both realizations of a pair: own angles ph, the
+// four neighbours' angles v, Philox block w; returns the angles to store and
+// adds the energy changes to ao / al / au (own block, left and upper
+// neighbour's block).
+template <typename S>
+__device__ __forceinline__ float2 update_entry(const Model& m, float2 ph, const float2 v[4],
+                                               uint32_t f, const uint32_t w[4], float2 beta,
+                                               float2& ao, float2& al, float2& au) {
+    float2 nc[4], ns[4];
+    neighbour_field(m, v, f, nc, ns);
+    const float2 C = sum4(nc), Sn = sum4(ns);
+    const PairNew n = pair_update<S>(ph, C, Sn, u01_2(w[0], w[2]), u01_2(w[1], w[3]), beta, m);
+    if (f & (EDGE_L | EDGE_U)) {
+        // (the neighbours' cosines and sines again: see split_edge)
+        float2 lc, ls, uc, us;
+        sincos_2(__fmul2_rn(both(m.q), v[0]), ls, lc);
+        sincos_2(__fmul2_rn(both(m.q), v[2]), us, uc);
+        split_edge_2<S>(n, ph, f, C, Sn, lc, ls, uc, us, m, ao, al, au);
+    } else {
+        ao = __fadd2_rn(ao, n.dE);
+    }
+    return n.phi;
+}
+
+// The same in one realization of the pair (the other one does not run): its
+// angle ph, its neighbours' angles v, its two Philox words.
+template <typename S>
+__device__ __forceinline__ float update_entry_one(const Model& m, float ph, const float v[4],
+                                                  uint32_t f, uint32_t w0, uint32_t w1, float beta,
+                                                  float& ao, float& al, float& au) {
+    float nc[4], ns[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) __sincosf(m.q * v[d], &ns[d], &nc[d]);
+    if ((f & 0xFu) != 0xFu) {
+#pragma unroll
+        for (int d = 0; d < 4; ++d)
+            if (!(f & (NB_L << d))) nc[d] = ns[d] = 0.0f;
+    }
+    const float C = (nc[0] + nc[1]) + (nc[2] + nc[3]);
+    const float Sn = (ns[0] + ns[1]) + (ns[2] + ns[3]);
+    const SiteNew n = site_update<S>(ph, C, Sn, u01(w0), u01(w1), beta, m);
+    if (f & (EDGE_L | EDGE_U))
+        split_edge<S>(n, ph, f, C, Sn, nc[0], ns[0], nc[2], ns[2], m, ao, al, au);
+    else
+        ao += n.dE;
+    return n.phi;
 }
 
 __device__ __forceinline__ void pair_running(const SweepArgs& a, int b, int rl, bool& run0,
@@ -209,32 +343,61 @@ __device__ __forceinline__ void pair_running(const SweepArgs& a, int b, int rl, 
     }
 }
 
-// All gap sites of colour c in one item. wpi warps share the item (wi = this
-// warp's index among them): warp wi handles realization pair q = wi mod G/2,
-// and the wpi / (G/2) warps of a pair split the entries 32 at a time. The
-// next entry of a lane is loaded while the current one is updated. The
-// block's list puts its edge entries first, so the branch that splits an
-// edge move bond by bond diverges in the first 32 entries only. kCal: the
-// calibration's chains, whose two lanes of a pair may sit at different
-// temperatures (the trisection's two points, or the k-point section's lane r
-// at point r mod n_pts), as in sweep_flat.
-template <int G, typename S, bool kCal = false>
-__device__ __forceinline__ void sweep_item(const SweepArgs& a, int item, int wi, int wpi,
+// Clears the sums of the pair's realizations that do not run.
+__device__ __forceinline__ void drop_idle(bool run0, bool run1, float2& ao, float2& al,
+                                          float2& au) {
+    if (!run0) ao.x = al.x = au.x = 0.0f;
+    if (!run1) ao.y = al.y = au.y = 0.0f;
+}
+
+// The gap entries e, e + step, ... < e1 of one unit, by one lane; the next
+// list entry is loaded while the current one is updated. kAll: both
+// realizations run; else one that does not keeps its angles, and its sums are
+// cleared at the end.
+template <typename S, bool kAll>
+__device__ __forceinline__ void sweep_entries(const SweepArgs& a, int e, int e1, int step, S* own,
+                                              const S* oth, uint32_t ctr1, uint32_t rpair,
+                                              uint32_t key1, float2 beta, bool run0, bool run1,
+                                              float2& ao, float2& al, float2& au) {
+    const float* bs =
+        a.beta_site ? a.beta_site + (size_t)a.colour * a.g.H * a.g.Wh : nullptr;
+    uint4 nx = e < e1 ? a.list[e] : make_uint4(0u, 0u, 0u, 0u);
+    for (; e < e1; e += step) {
+        const uint4 en = nx;
+        if (e + step < e1) nx = a.list[e + step];
+        uint32_t w[4];
+        philox4x32_10_rk(en.z, ctr1, rpair, 0u, a.rng.rk0, key1, w);
+        S* po = own + 2 * (size_t)en.x;
+        const float2 ph = Store<S>::load2(po);
+        float2 v[4];
+        load_neighbours<S>(a.g, oth, en, v);
+        const float2 bt = bs ? both(bs[en.x]) : beta;
+        float2 out = update_entry<S>(a.m, ph, v, en.y, w, bt, ao, al, au);
+        if constexpr (!kAll) out = make_float2(run0 ? out.x : ph.x, run1 ? out.y : ph.y);
+        Store<S>::store2(po, out);
+    }
+    if constexpr (!kAll) drop_idle(run0, run1, ao, al, au);
+}
+
+// All gap sites of colour c of one unit: block b in realization pair p, by CW
+// warps that split its entries 32 at a time (cw: this warp's index among
+// them). The block's list puts its edge entries first, so the branch that
+// splits an edge move bond by bond diverges in the first 32 entries only.
+// kCal: the calibration's chains, whose two lanes of a pair may sit at
+// different temperatures (the trisection's two points, or the k-point
+// section's lane r at point r mod n_pts), as in sweep_flat.
+template <typename S, bool kCal = false, bool kAll = false>
+__device__ __forceinline__ void sweep_item(const SweepArgs& a, int b, int p, int cw, int CW,
                                            uint32_t ctr1) {
-    constexpr int NP = G / 2;
     const int lane = threadIdx.x & 31;
-    const int q = wi % NP, cw = wi / NP, CW = wpi / NP;
-    const size_t plane = (size_t)a.g.H * a.g.Wh;
-    const int c = a.colour, co = c ^ 1;
-    const int b = item / a.groups, grp = item - b * a.groups;
     const int e0 = a.start[b], e1 = a.start[b + 1];
     if (e0 >= e1) return;
-    const int rl = grp * G + 2 * q;
+    const int rl = 2 * p;
     bool run0, run1;
     pair_running(a, b, rl, run0, run1);
     if (!(run0 || run1)) return;
-    S* own = static_cast<S*>(a.ang) + (size_t)(grp * 2 + c) * plane * G + 2 * q;
-    const S* oth = static_cast<const S*>(a.ang) + (size_t)(grp * 2 + co) * plane * G + 2 * q;
+    S* own = static_cast<S*>(a.ang) + pair_plane(a.g, p, a.colour);
+    const S* oth = static_cast<const S*>(a.ang) + pair_plane(a.g, p, a.colour ^ 1);
     float beta = a.beta[b], beta_odd = beta;
     if constexpr (kCal) {
         if (a.beta_pts) {
@@ -244,50 +407,18 @@ __device__ __forceinline__ void sweep_item(const SweepArgs& a, int item, int wi,
             beta_odd = a.beta_odd[b];
         }
     }
-    const float J = a.m.J;
     const uint32_t rpair = (a.r_base + (uint32_t)rl) >> 1;
-    const int sl = slice_of(a.sl, b);
-    const int4 rc = slice_rect(a.sl, sl);
-    const uint32_t key1 = slice_key1(a.sl, sl);
-    float ao0 = 0.f, ao1 = 0.f, al0 = 0.f, al1 = 0.f, au0 = 0.f, au1 = 0.f;
-    const int step = CW * 32;
-    int e = e0 + cw * 32 + lane;
-    uint2 nx = e < e1 ? a.list[e] : make_uint2(0u, 0u);
-    for (; e < e1; e += step) {
-        const uint2 en = nx;
-        if (e + step < e1) nx = a.list[e + step];
-        const int y = en.x >> 16, x = en.x & 0xffff;
-        const uint32_t f = en.y;
-        const uint32_t hs = (uint32_t)y * (uint32_t)a.g.Wh + (uint32_t)(x >> 1);
-        uint32_t w[4];
-        philox4x32_10_rk(local_index(rc, y, x), ctr1, rpair, 0u, a.rng.rk0, key1, w);
-        const float2 ph = Store<S>::load2(own + (size_t)hs * G);
-        float nc0[4], ns0[4], nc1[4], ns1[4];
-        neighbour_field<S>(a, oth, G, hs, x, f, nc0, ns0, nc1, ns1);
-        const float C0 = (nc0[0] + nc0[1]) + (nc0[2] + nc0[3]);
-        const float S0 = (ns0[0] + ns0[1]) + (ns0[2] + ns0[3]);
-        const float C1 = (nc1[0] + nc1[1]) + (nc1[2] + nc1[3]);
-        const float S1 = (ns1[0] + ns1[1]) + (ns1[2] + ns1[3]);
-        const float bt = a.beta_site ? a.beta_site[(size_t)y * a.g.W + x] : beta;
-        float2 out = ph;
-        if (run0) {
-            const SiteNew n = site_update<S>(ph.x, C0, S0, u01(w[0]), u01(w[1]), bt, a.m);
-            out.x = n.phi;
-            add_energy(n, f, C0, S0, nc0, ns0, J, ao0, al0, au0);
-        }
-        if (run1) {
-            const SiteNew n = site_update<S>(ph.y, C1, S1, u01(w[2]), u01(w[3]),
-                                             kCal ? beta_odd : bt, a.m);
-            out.y = n.phi;
-            add_energy(n, f, C1, S1, nc1, ns1, J, ao1, al1, au1);
-        }
-        Store<S>::store2(own + (size_t)hs * G, out);
-    }
+    const uint32_t key1 = slice_key1(a.sl, slice_of(a.sl, b));
+    float2 ao = both(0.0f), al = ao, au = ao;
+    const int e = e0 + cw * 32 + lane, step = CW * 32;
+    const float2 bt = make_float2(beta, beta_odd);
+    sweep_entries<S, kAll>(a, e, e1, step, own, oth, ctr1, rpair, key1, bt, run0, run1, ao, al,
+                           au);
     if (!a.energy) return;
     double* ea = a.eacc + (size_t)b * a.Rp + rl;
-    flush_pair(ea, ao0, ao1);
-    flush_pair(ea - a.Rp, al0, al1);
-    flush_pair(ea - (size_t)a.g.nbx * a.Rp, au0, au1);
+    flush_pair(ea, ao.x, ao.y);
+    flush_pair(ea - a.Rp, al.x, al.y);
+    flush_pair(ea - (size_t)a.g.nbx * a.Rp, au.x, au.y);
 }
 
 // Energy flush of one half-warp's unit: the FP32 sum over its 16 lanes, added
@@ -310,70 +441,36 @@ __device__ __forceinline__ void flush_pair_half(double* ea, float v0, float v1, 
 // colour holds few entries (about 64 at l_b = 16 and half the sites missing)
 // the last, partial pass wastes fewer lanes, and the warp's per-unit work
 // (bounds, flags, energy sums) serves two units. have: this half has a unit
-// (item, pair q within its lane group); every lane of the warp calls this.
-template <int G, typename S>
-__device__ __forceinline__ void sweep_item_half(const SweepArgs& a, int item, int q, bool have,
+// (block b, pair p); every lane of the warp calls this.
+template <typename S>
+__device__ __forceinline__ void sweep_item_half(const SweepArgs& a, int b, int p, bool have,
                                                 uint32_t ctr1) {
     const int hl = threadIdx.x & 15;
-    const size_t plane = (size_t)a.g.H * a.g.Wh;
-    const int c = a.colour, co = c ^ 1;
-    const int b = have ? item / a.groups : 0, grp = have ? item - b * a.groups : 0;
     int e0 = 0, e1 = 0;
     bool run0 = false, run1 = false;
-    const int rl = grp * G + 2 * q;
+    const int rl = 2 * p;
     if (have) {
         e0 = a.start[b];
         e1 = a.start[b + 1];
         pair_running(a, b, rl, run0, run1);
     }
     const bool act = have && e0 < e1 && (run0 || run1);
-    float ao0 = 0.f, ao1 = 0.f, al0 = 0.f, al1 = 0.f, au0 = 0.f, au1 = 0.f;
+    float2 ao = both(0.0f), al = ao, au = ao;
     if (act) {
-        S* own = static_cast<S*>(a.ang) + (size_t)(grp * 2 + c) * plane * G + 2 * q;
-        const S* oth = static_cast<const S*>(a.ang) + (size_t)(grp * 2 + co) * plane * G + 2 * q;
+        S* own = static_cast<S*>(a.ang) + pair_plane(a.g, p, a.colour);
+        const S* oth = static_cast<const S*>(a.ang) + pair_plane(a.g, p, a.colour ^ 1);
         const float beta = a.beta[b];
-        const float J = a.m.J;
         const uint32_t rpair = (a.r_base + (uint32_t)rl) >> 1;
-        const int sl = slice_of(a.sl, b);
-        const int4 rc = slice_rect(a.sl, sl);
-        const uint32_t key1 = slice_key1(a.sl, sl);
-        int e = e0 + hl;
-        uint2 nx = e < e1 ? a.list[e] : make_uint2(0u, 0u);
-        for (; e < e1; e += 16) {
-            const uint2 en = nx;
-            if (e + 16 < e1) nx = a.list[e + 16];
-            const int y = en.x >> 16, x = en.x & 0xffff;
-            const uint32_t f = en.y;
-            const uint32_t hs = (uint32_t)y * (uint32_t)a.g.Wh + (uint32_t)(x >> 1);
-            uint32_t w[4];
-            philox4x32_10_rk(local_index(rc, y, x), ctr1, rpair, 0u, a.rng.rk0, key1, w);
-            const float2 ph = Store<S>::load2(own + (size_t)hs * G);
-            float nc0[4], ns0[4], nc1[4], ns1[4];
-            neighbour_field<S>(a, oth, G, hs, x, f, nc0, ns0, nc1, ns1);
-            const float C0 = (nc0[0] + nc0[1]) + (nc0[2] + nc0[3]);
-            const float S0 = (ns0[0] + ns0[1]) + (ns0[2] + ns0[3]);
-            const float C1 = (nc1[0] + nc1[1]) + (nc1[2] + nc1[3]);
-            const float S1 = (ns1[0] + ns1[1]) + (ns1[2] + ns1[3]);
-            const float bt = a.beta_site ? a.beta_site[(size_t)y * a.g.W + x] : beta;
-            float2 out = ph;
-            if (run0) {
-                const SiteNew n = site_update<S>(ph.x, C0, S0, u01(w[0]), u01(w[1]), bt, a.m);
-                out.x = n.phi;
-                add_energy(n, f, C0, S0, nc0, ns0, J, ao0, al0, au0);
-            }
-            if (run1) {
-                const SiteNew n = site_update<S>(ph.y, C1, S1, u01(w[2]), u01(w[3]), bt, a.m);
-                out.y = n.phi;
-                add_energy(n, f, C1, S1, nc1, ns1, J, ao1, al1, au1);
-            }
-            Store<S>::store2(own + (size_t)hs * G, out);
-        }
+        const uint32_t key1 = slice_key1(a.sl, slice_of(a.sl, b));
+        // (one loop for both: the two halves of a warp would take turns in two)
+        sweep_entries<S, false>(a, e0 + hl, e1, 16, own, oth, ctr1, rpair, key1, both(beta), run0,
+                                run1, ao, al, au);
     }
     if (!a.energy) return;
     double* ea = a.eacc + (size_t)b * a.Rp + rl;
-    flush_pair_half(ea, ao0, ao1, act);
-    flush_pair_half(ea - a.Rp, al0, al1, act);
-    flush_pair_half(ea - (size_t)a.g.nbx * a.Rp, au0, au1, act);
+    flush_pair_half(ea, ao.x, ao.y, act);
+    flush_pair_half(ea - a.Rp, al.x, al.y, act);
+    flush_pair_half(ea - (size_t)a.g.nbx * a.Rp, au.x, au.y, act);
 }
 
 // One half-step over the whole list of one colour, flat: one thread per
@@ -415,17 +512,15 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
     const int b0 = (int)(a.list[t0 / NP].y >> META_SHIFT);
     const bool live = e < n_list;
     const int rl = grp * G + 2 * q;
-    uint2 en = make_uint2(0u, 0u);
+    uint4 en = make_uint4(0u, 0u, 0u, 0u);
     int b = b0;
     uint32_t w[4] = {0u, 0u, 0u, 0u};
     float beta = 0.0f, beta1 = 0.0f;
     if (live) {
         en = a.list[e];
         b = (int)(en.y >> META_SHIFT);
-        const int y = en.x >> 16, x = en.x & 0xffff;
-        const int sl = slice_of(a.sl, b);
-        philox4x32_10_rk(local_index(slice_rect(a.sl, sl), y, x), ctr1,
-                         (a.r_base + (uint32_t)rl) >> 1, 0u, a.rng.rk0, slice_key1(a.sl, sl), w);
+        philox4x32_10_rk(en.z, ctr1, (a.r_base + (uint32_t)rl) >> 1, 0u, a.rng.rk0,
+                         slice_key1(a.sl, slice_of(a.sl, b)), w);
         if (a.beta_pts) {
             beta = a.beta_pts[(size_t)(rl % a.n_pts) * a.g.nblk + b];
             beta1 = a.beta_pts[(size_t)((rl + 1) % a.n_pts) * a.g.nblk + b];
@@ -436,40 +531,31 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
     }
     grid_dep_wait();
     __syncthreads();
-    float ao0 = 0.f, ao1 = 0.f, al0 = 0.f, al1 = 0.f, au0 = 0.f, au1 = 0.f;
+    float2 ao = both(0.0f), al = ao, au = ao;
     uint32_t f = 0;
     if (live) {
-        const size_t plane = (size_t)a.g.H * a.g.Wh;
-        const int c = a.colour, co = c ^ 1;
         bool run0, run1;
         pair_running(a, b, rl, run0, run1);
         if (run0 || run1) {
-            float2* own = reinterpret_cast<float2*>(static_cast<float*>(a.ang) + (size_t)(grp * 2 + c) * plane * G) + q;
-            const float2* oth =
-                reinterpret_cast<const float2*>(static_cast<const float*>(a.ang) + (size_t)(grp * 2 + co) * plane * G) + q;
-            const int y = en.x >> 16, x = en.x & 0xffff;
             f = en.y;
-            const uint32_t hs = (uint32_t)y * (uint32_t)a.g.Wh + (uint32_t)(x >> 1);
-            const float2 ph = own[(size_t)hs * NP];
-            float nc0[4], ns0[4], nc1[4], ns1[4];
-            neighbour_field<float>(a, reinterpret_cast<const float*>(oth), G, hs, x, f, nc0, ns0,
-                                   nc1, ns1);
-            const float C0 = (nc0[0] + nc0[1]) + (nc0[2] + nc0[3]);
-            const float S0 = (ns0[0] + ns0[1]) + (ns0[2] + ns0[3]);
-            const float C1 = (nc1[0] + nc1[1]) + (nc1[2] + nc1[3]);
-            const float S1 = (ns1[0] + ns1[1]) + (ns1[2] + ns1[3]);
-            float2 out = ph;
-            if (run0) {
-                const SiteNew n = site_update<float>(ph.x, C0, S0, u01(w[0]), u01(w[1]), beta, a.m);
-                out.x = n.phi;
-                add_energy(n, f, C0, S0, nc0, ns0, a.m.J, ao0, al0, au0);
+            float* po = static_cast<float*>(a.ang) + pair_plane(a.g, rl >> 1, a.colour) +
+                        2 * (size_t)en.x;
+            const float* oth =
+                static_cast<const float*>(a.ang) + pair_plane(a.g, rl >> 1, a.colour ^ 1);
+            float2 v[4];
+            load_neighbours<float>(a.g, oth, en, v);
+            if (run0 && run1) {
+                Store<float>::store2(po, update_entry<float>(a.m, Store<float>::load2(po), v, f, w,
+                                                             make_float2(beta, beta1), ao, al, au));
+            } else {
+                // one lane runs (a bisection's single chain): the other's arithmetic left out
+                const int o = run0 ? 0 : 1;
+                const float v1[4] = {run0 ? v[0].x : v[0].y, run0 ? v[1].x : v[1].y,
+                                     run0 ? v[2].x : v[2].y, run0 ? v[3].x : v[3].y};
+                po[o] = update_entry_one<float>(a.m, po[o], v1, f, w[2 * o], w[2 * o + 1],
+                                                run0 ? beta : beta1, run0 ? ao.x : ao.y,
+                                                run0 ? al.x : al.y, run0 ? au.x : au.y);
             }
-            if (run1) {
-                const SiteNew n = site_update<float>(ph.y, C1, S1, u01(w[2]), u01(w[3]), beta1, a.m);
-                out.y = n.phi;
-                add_energy(n, f, C1, S1, nc1, ns1, a.m.J, ao1, al1, au1);
-            }
-            own[(size_t)hs * NP] = out;
         }
     }
     if (!a.energy) return;
@@ -480,39 +566,39 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
     if (__all_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, 0))) {
 #pragma unroll
         for (int d = 16; d >= NP; d >>= 1) {
-            ao0 += __shfl_xor_sync(0xffffffffu, ao0, d);
-            ao1 += __shfl_xor_sync(0xffffffffu, ao1, d);
+            ao.x += __shfl_xor_sync(0xffffffffu, ao.x, d);
+            ao.y += __shfl_xor_sync(0xffffffffu, ao.y, d);
         }
         if (lane < NP) {
             const int loc = b - b0;
             if (loc < kFlatBlocks) {
-                if (ao0 != 0.0f) atomicAdd(&acc[loc * G + 2 * lane], ao0);
-                if (ao1 != 0.0f) atomicAdd(&acc[loc * G + 2 * lane + 1], ao1);
+                if (ao.x != 0.0f) atomicAdd(&acc[loc * G + 2 * lane], ao.x);
+                if (ao.y != 0.0f) atomicAdd(&acc[loc * G + 2 * lane + 1], ao.y);
             } else {
                 double* ea = a.eacc + (size_t)b * a.Rp + grp * G + 2 * lane;
-                if (ao0 != 0.0f) atomicAdd(ea, (double)ao0);
-                if (ao1 != 0.0f) atomicAdd(ea + 1, (double)ao1);
+                if (ao.x != 0.0f) atomicAdd(ea, (double)ao.x);
+                if (ao.y != 0.0f) atomicAdd(ea + 1, (double)ao.y);
             }
         }
     } else if (live) {
         const int loc = b - b0;
         if (loc < kFlatBlocks) {
-            if (ao0 != 0.0f) atomicAdd(&acc[loc * G + 2 * q], ao0);
-            if (ao1 != 0.0f) atomicAdd(&acc[loc * G + 2 * q + 1], ao1);
+            if (ao.x != 0.0f) atomicAdd(&acc[loc * G + 2 * q], ao.x);
+            if (ao.y != 0.0f) atomicAdd(&acc[loc * G + 2 * q + 1], ao.y);
         } else {
             double* ea = a.eacc + (size_t)b * a.Rp + rl;
-            if (ao0 != 0.0f) atomicAdd(ea, (double)ao0);
-            if (ao1 != 0.0f) atomicAdd(ea + 1, (double)ao1);
+            if (ao.x != 0.0f) atomicAdd(ea, (double)ao.x);
+            if (ao.y != 0.0f) atomicAdd(ea + 1, (double)ao.y);
         }
     }
     // Left / up bonds of edge sites belong to the neighbouring blocks.
     if (f & (EDGE_L | EDGE_U)) {
         double* ea = a.eacc + (size_t)b * a.Rp + rl;
-        if (al0 != 0.0f) atomicAdd(ea - a.Rp, (double)al0);
-        if (al1 != 0.0f) atomicAdd(ea - a.Rp + 1, (double)al1);
+        if (al.x != 0.0f) atomicAdd(ea - a.Rp, (double)al.x);
+        if (al.y != 0.0f) atomicAdd(ea - a.Rp + 1, (double)al.y);
         const size_t up = (size_t)a.g.nbx * a.Rp;
-        if (au0 != 0.0f) atomicAdd(ea - up, (double)au0);
-        if (au1 != 0.0f) atomicAdd(ea - up + 1, (double)au1);
+        if (au.x != 0.0f) atomicAdd(ea - up, (double)au.x);
+        if (au.y != 0.0f) atomicAdd(ea - up + 1, (double)au.y);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kFlatBlocks * G; i += kFlatThreads) {
@@ -526,27 +612,27 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
 // 1 counts all bonds of its gap sites, colour 0 only those to sample
 // neighbours). Each lane sums its few bonds in FP32; the warp sums and the
 // block totals are FP64.
-template <int G, typename S>
-__device__ __forceinline__ void energy_item(const SweepArgs& a, int item, int wi, int wpi) {
-    constexpr int NP = G / 2;
+// The FP32 partial sums of the lanes depend on how the warps
+// split the entries: warp wi of a block's four takes pair wi mod NP of lane
+// group grp, and the 4 / NP warps of a pair split them 32 at a time.
+template <typename S>
+__device__ __forceinline__ void energy_item(const SweepArgs& a, int b, int grp, int NP, int wi,
+                                            int wpi) {
     const int lane = threadIdx.x & 31;
     const int q = wi % NP, cw = wi / NP, CW = wpi / NP;
-    const size_t plane = (size_t)a.g.H * a.g.Wh;
-    const int c = a.colour, co = c ^ 1;
-    const int b = item / a.groups, grp = item - b * a.groups;
-    const int rl = grp * G + 2 * q;
+    const int c = a.colour;
+    const int rl = 2 * (grp * NP + q);
     const int e0 = a.start[b], e1 = a.start[b + 1];
-    const S* own = static_cast<const S*>(a.ang) + (size_t)(grp * 2 + c) * plane * G + 2 * q;
-    const S* oth = static_cast<const S*>(a.ang) + (size_t)(grp * 2 + co) * plane * G + 2 * q;
+    const S* own = static_cast<const S*>(a.ang) + pair_plane(a.g, rl >> 1, c);
+    const S* oth = static_cast<const S*>(a.ang) + pair_plane(a.g, rl >> 1, c ^ 1);
     float o0 = 0.f, o1 = 0.f, l0 = 0.f, l1 = 0.f, u0 = 0.f, u1 = 0.f;
     for (int e = e0 + cw * 32 + lane; e < e1; e += CW * 32) {
-        const uint2 en = a.list[e];
-        const int y = en.x >> 16, x = en.x & 0xffff;
+        const uint4 en = a.list[e];
         const uint32_t f = en.y;
-        const uint32_t hs = (uint32_t)y * (uint32_t)a.g.Wh + (uint32_t)(x >> 1);
-        const float2 ph = Store<S>::load2(own + (size_t)hs * G);
-        float nc0[4], ns0[4], nc1[4], ns1[4];
-        neighbour_field<S>(a, oth, G, hs, x, f, nc0, ns0, nc1, ns1);
+        const float2 ph = Store<S>::load2(own + 2 * (size_t)en.x);
+        float2 v[4], nc[4], ns[4];
+        load_neighbours<S>(a.g, oth, en, v);
+        neighbour_field(a.m, v, f, nc, ns);
         float s0, c0, s1, c1;
         __sincosf(a.m.q * ph.x, &s0, &c0);
         __sincosf(a.m.q * ph.y, &s1, &c1);
@@ -554,8 +640,8 @@ __device__ __forceinline__ void energy_item(const SweepArgs& a, int item, int wi
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
             if (!((f & (NB_L << d)) && (take & (1u << d)))) continue;
-            const float b0 = -a.m.J * (c0 * nc0[d] + s0 * ns0[d]);
-            const float b1 = -a.m.J * (c1 * nc1[d] + s1 * ns1[d]);
+            const float b0 = -a.m.J * (c0 * nc[d].x + s0 * ns[d].x);
+            const float b1 = -a.m.J * (c1 * nc[d].y + s1 * ns[d].y);
             if (d == 0 && (f & EDGE_L)) { l0 += b0; l1 += b1; }
             else if (d == 2 && (f & EDGE_U)) { u0 += b0; u1 += b1; }
             else { o0 += b0; o1 += b1; }

@@ -10,7 +10,7 @@
 // another slice) stages zeros. Each staged value is then read by up to four
 // gap sites of the tile's own colour, which walk the tile's compacted gap
 // list, one thread per (gap site, realization pair). The arithmetic of an
-// update is that of the other half-step forms (site_update, add_energy_lu),
+// update is that of the other half-step forms (pair_update, split_edge_2),
 // on the same random numbers, so the forms agree bit for bit up to the order
 // of the FP32 energy sums.
 #include <cuda_bf16.h>
@@ -186,8 +186,10 @@ __global__ void __launch_bounds__(kTileThreads, 8) k_sweep_tile(SweepArgs a) {
         }
         if (rb == 0) continue;
         const TileFrame tf = tile_frame(g, tl, a.sl.of_block, tile);
-        const S* oth = static_cast<const S*>(a.ang) + (size_t)(grp * 2 + co) * plane * G;
-        S* own = static_cast<S*>(a.ang) + (size_t)(grp * 2 + c) * plane * G;
+        // (a thread keeps its pair through the tile: kTileThreads is a multiple of 4)
+        const int p = grp * (G / 2) + (threadIdx.x & 3);
+        const S* oth = static_cast<const S*>(a.ang) + pair_plane(g, p, co);
+        S* own = static_cast<S*>(a.ang) + pair_plane(g, p, c);
 
         // Stage: (cos, sin) of q phi_j for every realization of each running
         // pair, at every other-colour site of the tile and its halo.
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(kTileThreads, 8) k_sweep_tile(SweepArgs a) {
             float v = -1.0f;
             if (ok) v = stab[hs];
             float2 ang = make_float2(v, v);
-            if (v != v) ang = Store<S>::load2(oth + hs * G + 2 * q);
+            if (v != v) ang = Store<S>::load2(oth + 2 * hs);
             float s0, c0, s1, c1;
             __sincosf(q_m * ang.x, &s0, &c0);
             __sincosf(q_m * ang.y, &s1, &c1);
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(kTileThreads, 8) k_sweep_tile(SweepArgs a) {
         const int sl = slice_of(a.sl, b);
         const int4 rc = slice_rect(a.sl, sl);
         const uint32_t key1 = slice_key1(a.sl, sl);
-        float ao0 = 0.f, ao1 = 0.f, al0 = 0.f, al1 = 0.f, au0 = 0.f, au1 = 0.f;
+        float2 ao = both(0.0f), al = ao, au = ao;
         const int ne = e1 - e0;
         const int ncol = tf.ncol;
         for (int i = threadIdx.x; i < ne * 4; i += kTileThreads) {
@@ -240,37 +242,38 @@ __global__ void __launch_bounds__(kTileThreads, 8) k_sweep_tile(SweepArgs a) {
             const float4 R = stage[(r * ncol + kr) * 4 + q];
             const float4 U = stage[((r - 1) * ncol + hc) * 4 + q];
             const float4 D = stage[((r + 1) * ncol + hc) * 4 + q];
-            const float C0 = (L.x + R.x) + (U.x + D.x);
-            const float S0 = (L.y + R.y) + (U.y + D.y);
-            const float C1 = (L.z + R.z) + (U.z + D.z);
-            const float S1 = (L.w + R.w) + (U.w + D.w);
+            const float2 C = make_float2((L.x + R.x) + (U.x + D.x), (L.z + R.z) + (U.z + D.z));
+            const float2 Sn = make_float2((L.y + R.y) + (U.y + D.y), (L.w + R.w) + (U.w + D.w));
             const uint32_t hs = (uint32_t)y * (uint32_t)g.Wh + (uint32_t)(x >> 1);
-            S* po = own + (size_t)hs * G + 2 * q;
+            S* po = own + 2 * (size_t)hs;
             const float2 ph = Store<S>::load2(po);
             const int rl = grp * G + 2 * q;
             uint32_t w[4];
             philox4x32_10_rk(local_index(rc, y, x), ctr1, (a.r_base + (uint32_t)rl) >> 1, 0u,
                              a.rng.rk0, key1, w);
-            const float bt = a.beta_site ? a.beta_site[(size_t)y * g.W + x] : beta;
-            float2 out = ph;
-            if (run0) {
-                const SiteNew n = site_update<S>(ph.x, C0, S0, u01(w[0]), u01(w[1]), bt, a.m);
-                out.x = n.phi;
-                add_energy_lu(n, f, C0, S0, L.x, L.y, U.x, U.y, J, ao0, al0, au0);
-            }
-            if (run1) {
-                const SiteNew n = site_update<S>(ph.y, C1, S1, u01(w[2]), u01(w[3]), bt, a.m);
-                out.y = n.phi;
-                add_energy_lu(n, f, C1, S1, L.z, L.w, U.z, U.w, J, ao1, al1, au1);
-            }
+            const float bt = a.beta_site ? a.beta_site[(size_t)c * plane + hs] : beta;
+            const PairNew n = pair_update<S>(ph, C, Sn, u01_2(w[0], w[2]), u01_2(w[1], w[3]),
+                                             both(bt), a.m);
+            if (f & (EDGE_L | EDGE_U))
+                split_edge_2<S>(n, ph, f, C, Sn, make_float2(L.x, L.z), make_float2(L.y, L.w),
+                                make_float2(U.x, U.z), make_float2(U.y, U.w), a.m, ao, al, au);
+            else ao = __fadd2_rn(ao, n.dE);
+            // (a realization that does not run keeps its angle; drop_idle clears its sums)
+            const float2 out = make_float2(run0 ? n.phi.x : ph.x, run1 ? n.phi.y : ph.y);
             Store<S>::store2(po, out);
+        }
+
+        {
+            const int q = threadIdx.x & 3;
+            drop_idle(((rb >> (16 * q)) & 0xffull) != 0, ((rb >> (16 * q + 8)) & 0xffull) != 0, ao,
+                      al, au);
         }
 
         // The tile's energy changes: FP32 sums over the lanes of one pair
         // (lanes q, q + 4, ...) and over the warps, then one FP64 atomic per
         // (block, realization) for the own, left and upper blocks.
         if (a.energy) {
-            float v[6] = {ao0, ao1, al0, al1, au0, au1};
+            float v[6] = {ao.x, ao.y, al.x, al.y, au.x, au.y};
 #pragma unroll
             for (int d = 4; d < 32; d <<= 1)
 #pragma unroll
