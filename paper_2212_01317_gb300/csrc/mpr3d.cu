@@ -7,13 +7,14 @@
 // back-transformed.
 //
 // Layout: site (z, y, x), index i = (z H + y) W + x, colour (x + y + z) mod 2,
-// half-lattice state [colour][D][H][ceil(W/2)][pairs] of float2 (a
-// realization pair per element; sample angles in every lane); gap lists per
-// colour, block-major, of (site index, block). A thread updates one gap
-// site for one realization pair. Every site owns its +x, +y, +z bonds; a
-// site on the low x / y / z face of its block hands that bond's change to
-// the neighbouring block. The stop and calibration bookkeeping (per block
-// and realization) are the 2-D kernels.
+// half-lattice state [pair][colour][D][H][ceil(W/2)] of float2 (a realization
+// pair per element, a plane per pair and colour; sample angles in both lanes;
+// a layer, a row and two half-sites readable before and after it); gap lists
+// per colour, block-major (see gap_item3). A thread updates one gap site for
+// one realization pair. Every site owns its +x, +y, +z bonds; a site on the
+// low x / y / z face of its block hands that bond's change to the neighbouring
+// block. The stop and calibration bookkeeping (per block and realization) are
+// the 2-D kernels.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -29,6 +30,8 @@
 #include "mpr_internal.h"
 #include "mpr_launch.h"
 #include "mpr_memory.h"
+#include "mpr_pdl.h"
+#include "mpr_stats.cuh"
 #include "mpr_sweep.cuh"
 
 using namespace mpr;
@@ -43,9 +46,35 @@ __device__ __forceinline__ int block3(const Geom3& g, int z, int y, int x) {
     return ((z / g.lb) * g.nby + y / g.lb) * g.nbx + x / g.lb;
 }
 
-// Element (pair p) of site (z, y, x) in the half-lattice of its colour.
-__device__ __forceinline__ size_t hidx3(const Geom3& g, int c, int z, int y, int x, int np) {
-    return ((((size_t)c * g.D + z) * g.H + y) * g.Wh + (x >> 1)) * np;
+// Half index of site (z, y, x), and element offset of pair p's plane of colour c.
+__device__ __forceinline__ size_t half3(const Geom3& g, int z, int y, int x) {
+    return ((size_t)z * g.H + y) * g.Wh + (x >> 1);
+}
+__host__ __device__ inline size_t plane3(const Geom3& g, int p, int c) {
+    return ((size_t)p * 2 + (size_t)c) * g.D * g.H * g.Wh;
+}
+// Elements before and after the state that a neighbour load may touch.
+inline size_t guard3(const Geom3& g) { return (size_t)g.H * g.Wh + g.Wh + 2; }
+
+// Low bits of a gap entry's .y: which of the neighbours -x, +x, -y, +y, -z, +z
+// exist, and whether the -x, -y, -z bond belongs to the neighbouring block.
+constexpr uint32_t ALL6 = 0x3Fu;
+constexpr int FACE_SHIFT = 6;
+
+// The list entry of gap site (z, y, x) of block b: .x = half index, .y =
+// b << META_SHIFT | flags, .z = site index (the Philox counter word), .w = the
+// -x neighbour's half index (the +x one's is one more). Worked out once here,
+// where the sweep would divide site indices by the grid's sides in 64 bits for
+// every realization pair of every update.
+__device__ __forceinline__ uint4 gap_item3(const Geom3& g, int b, int z, int y, int x) {
+    const uint32_t f = (uint32_t)(x > 0) | (uint32_t)(x + 1 < g.W) << 1 | (uint32_t)(y > 0) << 2 |
+                       (uint32_t)(y + 1 < g.H) << 3 | (uint32_t)(z > 0) << 4 |
+                       (uint32_t)(z + 1 < g.D) << 5 | (uint32_t)(x > 0 && x % g.lb == 0) << 6 |
+                       (uint32_t)(y > 0 && y % g.lb == 0) << 7 |
+                       (uint32_t)(z > 0 && z % g.lb == 0) << 8;
+    const uint32_t h = (uint32_t)half3(g, z, y, x);
+    return make_uint4(h, (uint32_t)b << META_SHIFT | f,
+                      (uint32_t)(((int64_t)z * g.H + y) * g.W + x), h + (uint32_t)(x & 1) - 1u);
 }
 
 __device__ __forceinline__ uint32_t f2ord3(float f) {
@@ -55,12 +84,19 @@ __device__ __forceinline__ uint32_t f2ord3(float f) {
 
 __global__ void k3_minmax(const float* __restrict__ values, const uint8_t* __restrict__ mask,
                           int64_t n, uint32_t* __restrict__ mm) {
+    uint32_t lo = 0xffffffffu, hi = 0u;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (mask[i]) continue;
         const uint32_t o = f2ord3(values[i]);
-        atomicMin(&mm[0], o);
-        atomicMax(&mm[1], o);
+        lo = min(lo, o);
+        hi = max(hi, o);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(&mm[0], lo);
+        atomicMax(&mm[1], hi);
     }
 }
 
@@ -75,18 +111,20 @@ __global__ void k3_layout(int64_t n, const float* __restrict__ values,
                        : (float)(6.283185307179586476925 * ((double)values[i] - zmin) / (zmax - zmin));
 }
 
-// Eq. 2 per block (one warp per block, FP64): owned sample-sample bonds, all
-// owned bonds, sample mean angle, gap counts per colour.
-__global__ void k3_block_stats(Geom3 g, const float* __restrict__ values,
-                               const uint8_t* __restrict__ mask, double zmin, double zmax,
-                               int degenerate, double q, double J, double* __restrict__ Es,
-                               int32_t* __restrict__ Nsp, int32_t* __restrict__ Nb,
-                               double* __restrict__ ssum, int32_t* __restrict__ nsamp,
-                               int32_t* __restrict__ ngap0, int32_t* __restrict__ ngap1) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= g.nblk) return;
-    const int bx = warp % g.nbx, by = (warp / g.nbx) % g.nby, bz = warp / (g.nbx * g.nby);
+// Eq. 2 per block (one CTA per block, FP64): owned sample-sample bonds, all
+// owned bonds, sample mean angle, gap counts per colour. A block holds
+// thousands of sites and a grid few blocks: with one warp per block the 512
+// blocks of a 128^3 grid kept 3.4 warps per SM (693 us).
+constexpr int kStatsWarps = 8;
+__global__ void __launch_bounds__(32 * kStatsWarps)
+k3_block_stats(Geom3 g, const float* __restrict__ values, const uint8_t* __restrict__ mask,
+               double zmin, double zmax, int degenerate, double q, double J,
+               double* __restrict__ Es, int32_t* __restrict__ Nsp, int32_t* __restrict__ Nb,
+               double* __restrict__ ssum, int32_t* __restrict__ nsamp,
+               int32_t* __restrict__ ngap0, int32_t* __restrict__ ngap1) {
+    const int b = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int bx = b % g.nbx, by = (b / g.nbx) % g.nby, bz = b / (g.nbx * g.nby);
     const int x0 = bx * g.lb, y0 = by * g.lb, z0 = bz * g.lb;
     const int x1 = min(g.W, x0 + g.lb), y1 = min(g.H, y0 + g.lb), z1 = min(g.D, z0 + g.lb);
     const int bw = x1 - x0, bh = y1 - y0, nsite = bw * bh * (z1 - z0);
@@ -94,7 +132,7 @@ __global__ void k3_block_stats(Geom3 g, const float* __restrict__ values,
     const int64_t HW = (int64_t)g.H * g.W;
     double es = 0.0, sm = 0.0;
     int nsp = 0, nb = 0, ns = 0, c0 = 0, c1 = 0;
-    for (int j = lane; j < nsite; j += 32) {
+    for (int j = threadIdx.x; j < nsite; j += 32 * kStatsWarps) {
         const int x = x0 + j % bw, y = y0 + (j / bw) % bh, z = z0 + j / (bw * bh);
         const int64_t i = z * HW + (int64_t)y * g.W + x;
         const bool gap = mask[i] != 0;
@@ -112,36 +150,46 @@ __global__ void k3_block_stats(Geom3 g, const float* __restrict__ values,
             ++nb;
             if (!gap && !mask[nbr[k]]) {
                 const double pj = ((double)values[nbr[k]] - zmin) * scale;
-                es += -J * cos(q * (pi - pj));
+                es += -J * cos_bond(q * (pi - pj));
                 ++nsp;
             }
         }
     }
+    __shared__ double s_d[kStatsWarps][2];
+    __shared__ int s_i[kStatsWarps][5];
+    int v[5] = {nsp, nb, ns, c0, c1};
     for (int d = 16; d > 0; d >>= 1) {
         es += __shfl_xor_sync(0xffffffffu, es, d);
         sm += __shfl_xor_sync(0xffffffffu, sm, d);
-        nsp += __shfl_xor_sync(0xffffffffu, nsp, d);
-        nb += __shfl_xor_sync(0xffffffffu, nb, d);
-        ns += __shfl_xor_sync(0xffffffffu, ns, d);
-        c0 += __shfl_xor_sync(0xffffffffu, c0, d);
-        c1 += __shfl_xor_sync(0xffffffffu, c1, d);
     }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] = __reduce_add_sync(0xffffffffu, v[k]);
     if (lane == 0) {
-        Es[warp] = es;
-        Nsp[warp] = nsp;
-        Nb[warp] = nb;
-        ssum[warp] = sm;
-        nsamp[warp] = ns;
-        ngap0[warp] = c0;
-        ngap1[warp] = c1;
+        s_d[warp][0] = es;
+        s_d[warp][1] = sm;
+        for (int k = 0; k < 5; ++k) s_i[warp][k] = v[k];
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kStatsWarps; ++w) {
+        es += s_d[w][0];
+        sm += s_d[w][1];
+        for (int k = 0; k < 5; ++k) v[k] += s_i[w][k];
+    }
+    Es[b] = es;
+    Nsp[b] = v[0];
+    Nb[b] = v[1];
+    ssum[b] = sm;
+    nsamp[b] = v[2];
+    ngap0[b] = v[3];
+    ngap1[b] = v[4];
 }
 
-// Gap lists, block-major (one warp per block): (site index, block id).
+// Gap lists, block-major, in site order (one warp per block).
 __global__ void k3_build_lists(Geom3 g, const uint8_t* __restrict__ mask,
                                const int32_t* __restrict__ start0,
-                               const int32_t* __restrict__ start1, uint2* __restrict__ list0,
-                               uint2* __restrict__ list1) {
+                               const int32_t* __restrict__ start1, uint4* __restrict__ list0,
+                               uint4* __restrict__ list1) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= g.nblk) return;
@@ -154,19 +202,19 @@ __global__ void k3_build_lists(Geom3 g, const uint8_t* __restrict__ mask,
     for (int j0 = 0; j0 < nsite; j0 += 32) {
         const int j = j0 + lane;
         bool take = false;
-        int c = 0;
-        int64_t i = 0;
+        int x = 0, y = 0, z = 0, c = 0;
         if (j < nsite) {
-            const int x = x0 + j % bw, y = y0 + (j / bw) % bh, z = z0 + j / (bw * bh);
-            i = z * HW + (int64_t)y * g.W + x;
-            take = mask[i] != 0;
+            x = x0 + j % bw;
+            y = y0 + (j / bw) % bh;
+            z = z0 + j / (bw * bh);
+            take = mask[z * HW + (int64_t)y * g.W + x] != 0;
             c = (x + y + z) & 1;
         }
         const unsigned m0 = __ballot_sync(0xffffffffu, take && c == 0);
         const unsigned m1 = __ballot_sync(0xffffffffu, take && c == 1);
         if (take) {
             const unsigned below = (1u << lane) - 1u;
-            const uint2 e = make_uint2((uint32_t)i, (uint32_t)warp);
+            const uint4 e = gap_item3(g, warp, z, y, x);
             if (c == 0) list0[o0 + __popc(m0 & below)] = e;
             else list1[o1 + __popc(m1 & below)] = e;
         }
@@ -178,11 +226,11 @@ __global__ void k3_build_lists(Geom3 g, const uint8_t* __restrict__ mask,
 struct Args3 {
     Geom3 g;
     Model m;
-    uint32_t key0, key1;
+    uint32_t rk0[10], key1;  // round keys of key word 0, key word 1
     int colour;
-    const uint2* list;
-    int64_t n_list;
-    float2* ang;             // [2][D][H][Wh][np]
+    const uint4* list;
+    int n_list;
+    float2* ang;             // [np][2][D][H][Wh]
     const float* beta;       // [nblk]
     const uint8_t* running;  // [nblk][Rp] or nullptr (every lane r < R)
     double* eacc;            // [nblk][Rp] FP64 per-sweep changes
@@ -191,206 +239,319 @@ struct Args3 {
     uint32_t pair_base;      // Philox counter word 2 of lane pair 0 (realization base / 2)
     uint32_t ctr1;           // t | tag << 16
     int energy;
+    int chunks;              // consecutive 32-entry chunks of the list per warp
 };
 
-// The six neighbours' angles of site (z, y, x) for one realization pair, and
-// which of them exist. Order: -x, +x, -y, +y, -z, +z.
-__device__ __forceinline__ void neighbours3(const Args3& a, int z, int y, int x, int p, float2 v[6],
-                                            bool ex[6]) {
-    const Geom3& g = a.g;
-    const int co = a.colour ^ 1;
-    ex[0] = x > 0;
-    ex[1] = x + 1 < g.W;
-    ex[2] = y > 0;
-    ex[3] = y + 1 < g.H;
-    ex[4] = z > 0;
-    ex[5] = z + 1 < g.D;
-    const int nz[6] = {z, z, z, z, z - 1, z + 1};
-    const int ny[6] = {y, y, y - 1, y + 1, y, y};
-    const int nx[6] = {x - 1, x + 1, x, x, x, x};
-#pragma unroll
-    for (int d = 0; d < 6; ++d)
-        v[d] = ex[d] ? a.ang[hidx3(g, co, nz[d], ny[d], nx[d], a.np) + p] : make_float2(0.f, 0.f);
+// The six neighbours' angles (-x, +x, -y, +y, -z, +z) for one realization
+// pair, from its plane of the other colour. One that does not exist reads some
+// other element or the state's guard; the caller drops it by the entry's flags.
+__device__ __forceinline__ void neighbours3(const Geom3& g, const float2* __restrict__ oth,
+                                            const uint4& en, float2 v[6]) {
+    const float2* left = oth + (ptrdiff_t)(int)en.w;
+    const float2* here = oth + en.x;
+    const ptrdiff_t layer = (ptrdiff_t)g.H * g.Wh;
+    v[0] = left[0];
+    v[1] = left[1];
+    v[2] = *(here - g.Wh);
+    v[3] = here[g.Wh];
+    v[4] = *(here - layer);
+    v[5] = here[layer];
 }
 
-// One half-step: thread per (gap entry of the colour, realization pair).
-__global__ void __launch_bounds__(256) k3_sweep(Args3 a) {
-    const Geom3& g = a.g;
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t e = t / a.np;
-    const int p = (int)(t % a.np);
-    const int lane = threadIdx.x & 31;
-    float ao0 = 0.f, ao1 = 0.f, ae[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    int b = -1;
-    if (e < a.n_list) {
-        const uint2 en = a.list[e];
-        b = (int)en.y;
-        const int64_t HW = (int64_t)g.H * g.W;
-        const int z = (int)(en.x / HW), y = (int)((en.x % HW) / g.W), x = (int)(en.x % g.W);
-        const int rl = 2 * p;
-        bool run0, run1;
-        if (a.running) {
-            run0 = a.running[(size_t)b * a.Rp + rl] != 0;
-            run1 = a.running[(size_t)b * a.Rp + rl + 1] != 0;
-        } else {
-            run0 = rl < a.R;
-            run1 = rl + 1 < a.R;
-        }
-        if (run0 || run1) {
-            uint32_t w[4];
-            philox4x32_10(en.x, a.ctr1, a.pair_base + (uint32_t)p, 0u, a.key0, a.key1, w);
-            float2 v[6];
-            bool ex[6];
-            neighbours3(a, z, y, x, p, v, ex);
-            float nc0[6], ns0[6], nc1[6], ns1[6];
-            float C0 = 0.f, S0 = 0.f, C1 = 0.f, S1 = 0.f;
-#pragma unroll
-            for (int d = 0; d < 6; ++d) {
-                const float mk = ex[d] ? 1.0f : 0.0f;
-                float s0, c0, s1, c1;
-                __sincosf(a.m.q * v[d].x, &s0, &c0);
-                __sincosf(a.m.q * v[d].y, &s1, &c1);
-                nc0[d] = mk * c0; ns0[d] = mk * s0; nc1[d] = mk * c1; ns1[d] = mk * s1;
-            }
-            C0 = ((nc0[0] + nc0[1]) + (nc0[2] + nc0[3])) + (nc0[4] + nc0[5]);
-            S0 = ((ns0[0] + ns0[1]) + (ns0[2] + ns0[3])) + (ns0[4] + ns0[5]);
-            C1 = ((nc1[0] + nc1[1]) + (nc1[2] + nc1[3])) + (nc1[4] + nc1[5]);
-            S1 = ((ns1[0] + ns1[1]) + (ns1[2] + ns1[3])) + (ns1[4] + ns1[5]);
-            const size_t h = hidx3(g, a.colour, z, y, x, a.np) + p;
-            const float2 ph = a.ang[h];
-            float2 out = ph;
-            const float beta = a.beta[b];
-            // faces of the block whose bond belongs to the neighbouring block
-            const bool edge[3] = {x > 0 && x % g.lb == 0, y > 0 && y % g.lb == 0,
-                                  z > 0 && z % g.lb == 0};
-            const float J = a.m.J;
-            if (run0) {
-                const SiteNew n = site_update<float>(ph.x, C0, S0, u01(w[0]), u01(w[1]), beta, a.m);
-                out.x = n.phi;
-                ao0 += n.dE;
-                if (edge[0] || edge[1] || edge[2]) {
-                    float co, so, ca, sa, cn, sn;
-                    __sincosf(a.m.q * ph.x, &so, &co);
-                    __sincosf(a.m.q * n.mid, &sa, &ca);
-                    final_cs(n.refl, ca, sa, C0, S0, cn, sn);
-                    const float dc = cn - co, ds = sn - so;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        if (edge[k]) {
-                            const float d = -J * (dc * nc0[2 * k] + ds * ns0[2 * k]);
-                            ao0 -= d;
-                            ae[k][0] += d;
-                        }
-                }
-            }
-            if (run1) {
-                const SiteNew n = site_update<float>(ph.y, C1, S1, u01(w[2]), u01(w[3]), beta, a.m);
-                out.y = n.phi;
-                ao1 += n.dE;
-                if (edge[0] || edge[1] || edge[2]) {
-                    float co, so, ca, sa, cn, sn;
-                    __sincosf(a.m.q * ph.y, &so, &co);
-                    __sincosf(a.m.q * n.mid, &sa, &ca);
-                    final_cs(n.refl, ca, sa, C1, S1, cn, sn);
-                    const float dc = cn - co, ds = sn - so;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        if (edge[k]) {
-                            const float d = -J * (dc * nc1[2 * k] + ds * ns1[2 * k]);
-                            ao1 -= d;
-                            ae[k][1] += d;
-                        }
-                }
-            }
-            a.ang[h] = out;
-        }
-    }
-    if (!a.energy) return;
-    // Block changes: one warp sum when every lane works on the same block
-    // and pair (block-major lists make that the common case), else atomics.
-    const int key = b < 0 ? -1 : b * a.np + p;
-    const int k0 = __shfl_sync(0xffffffffu, key, 0);
-    const bool uni = __all_sync(0xffffffffu, key == k0) && k0 >= 0;
-    const size_t off[4] = {0, 1, (size_t)g.nbx, (size_t)g.nbx * g.nby};
-    float vals[4][2] = {{ao0, ao1}, {ae[0][0], ae[0][1]}, {ae[1][0], ae[1][1]}, {ae[2][0], ae[2][1]}};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        float v0 = vals[k][0], v1 = vals[k][1];
-        if (uni) {
-            for (int d = 16; d > 0; d >>= 1) {
-                v0 += __shfl_xor_sync(0xffffffffu, v0, d);
-                v1 += __shfl_xor_sync(0xffffffffu, v1, d);
-            }
-            if (lane != 0) continue;
-        }
-        if (b < 0 || (v0 == 0.0f && v1 == 0.0f)) continue;
-        double* ea = a.eacc + ((size_t)b - off[k]) * a.Rp + 2 * p;
-        if (v0 != 0.0f) atomicAdd(ea, (double)v0);
-        if (v1 != 0.0f) atomicAdd(ea + 1, (double)v1);
-    }
+template <typename V> __device__ __forceinline__ V sum6(const V v[6]);
+template <> __device__ __forceinline__ float sum6(const float v[6]) {
+    return ((v[0] + v[1]) + (v[2] + v[3])) + (v[4] + v[5]);
+}
+template <> __device__ __forceinline__ float2 sum6(const float2 v[6]) {
+    return __fadd2_rn(__fadd2_rn(__fadd2_rn(v[0], v[1]), __fadd2_rn(v[2], v[3])),
+                      __fadd2_rn(v[4], v[5]));
 }
 
-// Block energies from scratch (FP64 atomics into ecur, which holds E_s,b):
-// colour 1 adds every bond of its gap sites, colour 0 only the bonds to
-// sample neighbours, each to the block that owns it.
-__global__ void k3_energy(Args3 a, const uint8_t* __restrict__ mask) {
-    const Geom3& g = a.g;
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t e = t / a.np;
-    const int p = (int)(t % a.np);
-    if (e >= a.n_list) return;
-    const uint2 en = a.list[e];
-    const int b = (int)en.y;
-    const int64_t HW = (int64_t)g.H * g.W;
-    const int z = (int)(en.x / HW), y = (int)((en.x % HW) / g.W), x = (int)(en.x % g.W);
+// A move on the block's low faces, bond by bond: what the neighbouring blocks
+// own goes to ae[k] (faces x, y, z) instead of ao. nc, ns: the neighbours'
+// (cos, sin). The roundings are spelled out (see bond_change).
+__device__ __forceinline__ void split_faces(const SiteNew& n, float phi, uint32_t f, float C,
+                                            float Sn, const float nc[3], const float ns[3],
+                                            const Model& m, float& ao, float ae[3]) {
+    float co, so, ca, sa, cn, sn;
+    __sincosf(m.q * phi, &so, &co);
+    __sincosf(m.q * n.mid, &sa, &ca);
+    final_cs(n.refl, ca, sa, C, Sn, cn, sn);
+    const float dc = cn - co, ds = sn - so;
+    ao += n.dE;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        if (f & (1u << (FACE_SHIFT + k))) {
+            const float d = bond_change<float>(dc, ds, nc[k], ns[k], m.J);
+            ao -= d;
+            ae[k] += d;
+        }
+}
+
+// One gap entry in both realizations of pair p (kOne: in the even one, the
+// only lane of a single-chain calibration): new angles stored, energy changes
+// into ao and, for the faces, ae.
+template <bool kOne>
+__device__ __forceinline__ void update3(const Args3& a, float2* own, const float2* oth,
+                                        const uint4& en, const uint32_t w[4], float beta, bool run0,
+                                        bool run1, float2& ao, float2 ae[3]) {
+    const uint32_t f = en.y;
+    const Model& m = a.m;
     float2 v[6];
-    bool ex[6];
-    neighbours3(a, z, y, x, p, v, ex);
-    const float2 ph = a.ang[hidx3(g, a.colour, z, y, x, a.np) + p];
-    const int64_t ni[6] = {-1, 1, -(int64_t)g.W, (int64_t)g.W, -HW, HW};
-    const size_t owner_off[6] = {1, 0, (size_t)g.nbx, 0, (size_t)g.nbx * g.nby, 0};
-    const bool face[6] = {x % g.lb == 0, false, y % g.lb == 0, false, z % g.lb == 0, false};
-    for (int d = 0; d < 6; ++d) {
-        if (!ex[d]) continue;
-        if (a.colour == 0 && mask[(int64_t)en.x + ni[d]]) continue;   // gap-gap bonds: colour 1
-        const double b0 = -a.m.J * cos((double)a.m.q * ((double)ph.x - (double)v[d].x));
-        const double b1 = -a.m.J * cos((double)a.m.q * ((double)ph.y - (double)v[d].y));
-        const size_t ob = (size_t)b - (face[d] ? owner_off[d] : 0);
-        atomicAdd(&a.ecur[ob * a.Rp + 2 * p], b0);
-        atomicAdd(&a.ecur[ob * a.Rp + 2 * p + 1], b1);
+    neighbours3(a.g, oth, en, v);
+    const float2 ph = own[en.x];
+    if constexpr (kOne) {
+        float nc[6], ns[6];
+#pragma unroll
+        for (int d = 0; d < 6; ++d) __sincosf(m.q * v[d].x, &ns[d], &nc[d]);
+        if ((f & ALL6) != ALL6) {
+#pragma unroll
+            for (int d = 0; d < 6; ++d)
+                if (!(f & (1u << d))) nc[d] = ns[d] = 0.0f;
+        }
+        const float C = sum6<float>(nc), Sn = sum6<float>(ns);
+        const SiteNew n = site_update<float>(ph.x, C, Sn, u01(w[0]), u01(w[1]), beta, m);
+        own[en.x].x = n.phi;
+        if (f & (7u << FACE_SHIFT)) {
+            const float lc[3] = {nc[0], nc[2], nc[4]}, ls[3] = {ns[0], ns[2], ns[4]};
+            float e[3] = {0.0f, 0.0f, 0.0f};
+            split_faces(n, ph.x, f, C, Sn, lc, ls, m, ao.x, e);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) ae[k].x = e[k];
+        } else {
+            ao.x += n.dE;
+        }
+    } else {
+        float2 nc[6], ns[6];
+#pragma unroll
+        for (int d = 0; d < 6; ++d) sincos_2(__fmul2_rn(both(m.q), v[d]), ns[d], nc[d]);
+        if ((f & ALL6) != ALL6) {
+#pragma unroll
+            for (int d = 0; d < 6; ++d)
+                if (!(f & (1u << d))) nc[d] = ns[d] = both(0.0f);
+        }
+        const float2 C = sum6<float2>(nc), Sn = sum6<float2>(ns);
+        const PairNew n = pair_update<float>(ph, C, Sn, u01_2(w[0], w[2]), u01_2(w[1], w[3]),
+                                             both(beta), m);
+        own[en.x] = make_float2(run0 ? n.phi.x : ph.x, run1 ? n.phi.y : ph.y);
+        float2 o = n.dE;
+        if (f & (7u << FACE_SHIFT)) {
+            o = both(0.0f);
+            float e0[3] = {0.0f, 0.0f, 0.0f}, e1[3] = {0.0f, 0.0f, 0.0f};
+            // (cosines and sines again, as in split_edge_2's callers)
+            float2 lc[3], ls[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sincos_2(__fmul2_rn(both(m.q), v[2 * k]), ls[k], lc[k]);
+            const float c0[3] = {lc[0].x, lc[1].x, lc[2].x}, s0[3] = {ls[0].x, ls[1].x, ls[2].x};
+            const float c1[3] = {lc[0].y, lc[1].y, lc[2].y}, s1[3] = {ls[0].y, ls[1].y, ls[2].y};
+            split_faces(SiteNew{n.phi.x, n.mid.x, n.dE.x, n.refl0}, ph.x, f, C.x, Sn.x, c0, s0, m,
+                        o.x, e0);
+            split_faces(SiteNew{n.phi.y, n.mid.y, n.dE.y, n.refl1}, ph.y, f, C.y, Sn.y, c1, s1, m,
+                        o.y, e1);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                ae[k] = make_float2(run0 ? e0[k] : 0.0f, run1 ? e1[k] : 0.0f);
+        }
+        ao = make_float2(run0 ? o.x : 0.0f, run1 ? o.y : 0.0f);
     }
 }
 
-// State: samples in every lane, gaps at their block's mean sample angle.
-__global__ void k3_init(Geom3 g, const float* __restrict__ phi_s, const uint8_t* __restrict__ mask,
-                        const float* __restrict__ init_angle, float2* __restrict__ ang, int np) {
+// FP64 warp sum of a pair's changes, added by lane 0.
+__device__ __forceinline__ void flush3(double* ea, double x, double y) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, d);
+        y += __shfl_xor_sync(0xffffffffu, y, d);
+    }
+    if ((threadIdx.x & 31) != 0) return;
+    if (x != 0.0) atomicAdd(ea, x);
+    if (y != 0.0) atomicAdd(ea + 1, y);
+}
+
+__device__ __forceinline__ void add3(double* ea, float2 v) {
+    if (v.x != 0.0f) atomicAdd(ea, (double)v.x);
+    if (v.y != 0.0f) atomicAdd(ea + 1, (double)v.y);
+}
+
+// FP32 warp sum of a pair's changes (kOne: of its even lane only).
+template <bool kOne> __device__ __forceinline__ float2 warp_sum3(float2 v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, d);
+        if constexpr (!kOne) v.y += __shfl_xor_sync(0xffffffffu, v.y, d);
+    }
+    return v;
+}
+
+// One half-step: a warp per run of consecutive 32-entry chunks of the colour's
+// list and realization pair (blockIdx.y), and f.ctas trailing CTAs that fold
+// the previous sweep of a calibration. The block sums: with several pairs every
+// update's change is summed in FP64 (per lane while the warp stays in a block,
+// then over the warp), with one pair a chunk's changes are an FP32 warp sum
+// added in FP64; a chunk that spans blocks adds lane by lane. One FP64 atomic
+// per block and warp instead of one per update. 128^3, half the sites missing,
+// l_b = 16: 20 realizations 43 -> 86 G updates/s, single-chain calibration 14 ->
+// 49 (10.7 us per half-step of 524 k updates), against 64-bit divisions of the
+// site index, pairs interleaved per site and an FP64 atomic per update. Bound
+// by instruction issue in large batches, by the latency of one chunk's chain in
+// a single-chain calibration. CTAs per SM: 9 of 6 to 9 for pairs, 10 of 8 to 16
+// for single chains.
+constexpr int kSweep3Threads = 128;
+template <bool kOne>
+__global__ void __launch_bounds__(kSweep3Threads, kOne ? 10 : 9) k3_sweep(Args3 a, FoldArgs f) {
+    grid_dep_launch();
+    const int ctas = (int)gridDim.x - f.ctas;
+    if ((int)blockIdx.x >= ctas) {
+        grid_dep_wait();
+        if (blockIdx.y == 0) fold_block_energies<kSweep3Threads>(f, (int)blockIdx.x - ctas);
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int p = blockIdx.y, rl = 2 * p;
+    const int c0 = ((int)blockIdx.x * (kSweep3Threads / 32) + (int)(threadIdx.x >> 5)) * a.chunks;
+    const int last = a.n_list - 1;
+    float2* own = a.ang + plane3(a.g, p, a.colour);
+    const float2* oth = a.ang + plane3(a.g, p, a.colour ^ 1);
+    const bool sum32 = a.np == 1;
+    double dx = 0.0, dy = 0.0;       // the lane's changes in block cur
+    int cur = -1;
+    if (c0 * 32 > last) {
+        grid_dep_wait();
+        return;
+    }
+    for (int k = 0; k < a.chunks; ++k) {
+        const int base = (c0 + k) * 32;
+        if (base > last) break;
+        const bool live = base + lane <= last;
+        const uint4 en = a.list[min(base + lane, last)];
+        const int b = (int)(en.y >> META_SHIFT);
+        uint32_t w[4];
+        philox4x32_10_rk(en.z, a.ctr1, a.pair_base + (uint32_t)p, 0u, a.rk0, a.key1, w);
+        const float beta = a.beta[b];
+        // (the entry, its Philox block and the temperature do not depend on
+        // the previous half-step)
+        if (k == 0) grid_dep_wait();
+        const int b0 = __shfl_sync(0xffffffffu, b, 0);
+        const bool one_block = __all_sync(0xffffffffu, live && b == b0);
+        bool run0 = live && rl < a.R, run1 = live && rl + 1 < a.R;
+        if (a.running) {
+            const uchar2 r2 =
+                *reinterpret_cast<const uchar2*>(a.running + (size_t)b * a.Rp + rl);
+            run0 = live && r2.x != 0;
+            run1 = live && r2.y != 0;
+        }
+        float2 ao = both(0.0f), ae[3] = {ao, ao, ao};
+        if (run0 || run1) {
+            update3<kOne>(a, own, oth, en, w, beta, run0, run1, ao, ae);
+        }
+        if (!a.energy) continue;
+        const size_t off[3] = {1, (size_t)a.g.nbx, (size_t)a.g.nbx * a.g.nby};
+        double* ea = a.eacc + (size_t)b * a.Rp + rl;
+        if (one_block && sum32) {
+            ao = warp_sum3<kOne>(ao);
+            if (lane == 0) add3(ea, ao);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                if (!__any_sync(0xffffffffu, (en.y & (1u << (FACE_SHIFT + j))) != 0)) continue;
+                const float2 s = warp_sum3<kOne>(ae[j]);
+                if (lane == 0) add3(ea - off[j] * a.Rp, s);
+            }
+            continue;
+        }
+        if (one_block) {
+            if (b0 != cur) {
+                if (cur >= 0) flush3(a.eacc + (size_t)cur * a.Rp + rl, dx, dy);
+                dx = dy = 0.0;
+                cur = b0;
+            }
+            dx += (double)ao.x;
+            dy += (double)ao.y;
+        } else {
+            add3(ea, ao);
+        }
+        if (en.y & (7u << FACE_SHIFT)) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) add3(ea - off[j] * a.Rp, ae[j]);
+        }
+    }
+    if (cur >= 0) flush3(a.eacc + (size_t)cur * a.Rp + rl, dx, dy);
+}
+
+// Block energies of the start state from scratch (FP64 into ecur, which holds
+// E_s,b): the bonds of the list entries [e0, e1) in pair blockIdx.y, whose two
+// lanes hold the same start. Colour 1 adds every bond of its gap sites, colour
+// 0 only the bonds to sample neighbours, each to the block that owns it.
+__global__ void k3_energy(Args3 a, const uint8_t* __restrict__ mask, int e0, int e1) {
+    const Geom3& g = a.g;
+    const int e = e0 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const bool live = e < e1;
+    const uint4 en = a.list[live ? e : e1 - 1];
+    const int b = (int)(en.y >> META_SHIFT);
+    const int64_t HW = (int64_t)g.H * g.W;
+    const size_t off[3] = {1, (size_t)g.nbx, (size_t)g.nbx * g.nby};
+    double* ecur = a.ecur + 2 * (size_t)blockIdx.y;
+    auto add = [&](size_t blk, double v) {
+        atomicAdd(&ecur[blk * a.Rp], v);
+        atomicAdd(&ecur[blk * a.Rp + 1], v);
+    };
+    double own = 0.0;
+    if (live) {
+        float2 v[6];
+        neighbours3(g, a.ang + plane3(g, blockIdx.y, a.colour ^ 1), en, v);
+        const float ph = a.ang[plane3(g, blockIdx.y, a.colour) + en.x].x;
+        const int64_t ni[6] = {-1, 1, -(int64_t)g.W, (int64_t)g.W, -HW, HW};
+#pragma unroll
+        for (int d = 0; d < 6; ++d) {
+            if (!(en.y & (1u << d))) continue;
+            if (a.colour == 0 && mask[(int64_t)en.z + ni[d]]) continue;   // gap-gap: colour 1
+            const double eb = -a.m.J * cos_bond((double)a.m.q * ((double)ph - (double)v[d].x));
+            if ((d & 1) == 0 && (en.y & (1u << (FACE_SHIFT + d / 2)))) add((size_t)b - off[d / 2], eb);
+            else own += eb;
+        }
+    }
+    const int b0 = __shfl_sync(0xffffffffu, b, 0);
+    if (__all_sync(0xffffffffu, b == b0)) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) own += __shfl_xor_sync(0xffffffffu, own, d);
+        if ((threadIdx.x & 31) != 0) own = 0.0;
+    }
+    if (own != 0.0) add(b, own);
+}
+
+// Sample angles into both lanes of every pair's planes (blockIdx.y: the pair).
+__global__ void k3_fill_samples(Geom3 g, const float* __restrict__ phi_s,
+                                const uint8_t* __restrict__ mask, float2* __restrict__ ang) {
     const int64_t n = (int64_t)g.D * g.H * g.W;
-    const int64_t HW = (int64_t)g.H * g.W;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n * np;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / np;
-        const int p = (int)(t % np);
-        const int z = (int)(i / HW), y = (int)((i % HW) / g.W), x = (int)(i % g.W);
-        const float v = mask[i] ? init_angle[block3(g, z, y, x)] : phi_s[i];
-        ang[hidx3(g, (x + y + z) & 1, z, y, x, np) + p] = make_float2(v, v);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        if (mask[i]) continue;
+        const uint32_t row = (uint32_t)i / (uint32_t)g.W;
+        const int x = (int)((uint32_t)i - row * (uint32_t)g.W);
+        const int z = (int)(row / (uint32_t)g.H), y = (int)(row - (uint32_t)z * (uint32_t)g.H);
+        ang[plane3(g, blockIdx.y, (x + y + z) & 1) + half3(g, z, y, x)] = both(phi_s[i]);
     }
 }
 
-__global__ void k3_accumulate(Geom3 g, const uint2* __restrict__ list, int64_t n_list, int colour,
-                              const float2* __restrict__ ang, int np, int R,
-                              double* __restrict__ sum) {
-    const int64_t HW = (int64_t)g.H * g.W;
+// Gap sites at their block's mean sample angle (blockIdx.y: the pair).
+__global__ void k3_init(Geom3 g, const uint4* __restrict__ list, int n_list, int colour,
+                        const float* __restrict__ init_angle, float2* __restrict__ ang) {
+    float2* dst = ang + plane3(g, blockIdx.y, colour);
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_list; e += gridDim.x * blockDim.x)
+        dst[list[e].x] = both(init_angle[list[e].y >> META_SHIFT]);
+}
+
+__global__ void k3_accumulate(Geom3 g, const uint4* __restrict__ list, int64_t n_list, int colour,
+                              const float2* __restrict__ ang, int R, double* __restrict__ sum) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_list;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = list[e].x;
-        const int z = (int)(i / HW), y = (int)((i % HW) / g.W), x = (int)(i % g.W);
-        const size_t h = hidx3(g, colour, z, y, x, np);
+        const uint4 en = list[e];
         double s = 0.0;
-        for (int r = 0; r < R; ++r) {
-            const float2 v = ang[h + r / 2];
-            s += (double)((r & 1) ? v.y : v.x);
+        for (int r = 0; r < R; r += 2) {
+            const float2 v = ang[plane3(g, r / 2, colour) + en.x];
+            s += (double)v.x;
+            if (r + 1 < R) s += (double)v.y;
         }
-        sum[i] += s;
+        sum[en.z] += s;
     }
 }
 
@@ -414,27 +575,27 @@ __global__ void k3_predict(int64_t n, const float* __restrict__ values,
     }
 }
 
-__global__ void k3_get_state(Geom3 g, const float2* __restrict__ ang, int np, int r,
+__global__ void k3_get_state(Geom3 g, const float2* __restrict__ ang, int r,
                              float* __restrict__ out) {
     const int64_t n = (int64_t)g.D * g.H * g.W;
     const int64_t HW = (int64_t)g.H * g.W;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int z = (int)(i / HW), y = (int)((i % HW) / g.W), x = (int)(i % g.W);
-        const float2 v = ang[hidx3(g, (x + y + z) & 1, z, y, x, np) + r / 2];
+        const float2 v = ang[plane3(g, r / 2, (x + y + z) & 1) + half3(g, z, y, x)];
         out[i] = (r & 1) ? v.y : v.x;
     }
 }
 
 __global__ void k3_set_state(Geom3 g, const uint8_t* __restrict__ mask, float2* __restrict__ ang,
-                             int np, int r, const float* __restrict__ in) {
+                             int r, const float* __restrict__ in) {
     const int64_t n = (int64_t)g.D * g.H * g.W;
     const int64_t HW = (int64_t)g.H * g.W;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (!mask[i]) continue;
         const int z = (int)(i / HW), y = (int)((i % HW) / g.W), x = (int)(i % g.W);
-        float2& v = ang[hidx3(g, (x + y + z) & 1, z, y, x, np) + r / 2];
+        float2& v = ang[plane3(g, r / 2, (x + y + z) & 1) + half3(g, z, y, x)];
         if (r & 1) v.y = in[i]; else v.x = in[i];
     }
 }
@@ -465,7 +626,7 @@ struct mpr3_ctx {
     int64_t n = 0, n_gap[2] = {0, 0};
     float *values = nullptr, *phi_s = nullptr, *init_angle = nullptr;
     uint8_t* mask = nullptr;
-    uint2* list[2] = {nullptr, nullptr};
+    uint4* list[2] = {nullptr, nullptr};
     int32_t* start[2] = {nullptr, nullptr};
     double *Es = nullptr, *es = nullptr, *inb = nullptr, *ssum = nullptr;
     int32_t *Nsp = nullptr, *Nb = nullptr, *nsamp = nullptr, *ngap = nullptr,
@@ -480,9 +641,11 @@ struct mpr3_ctx {
     int np = 0, R = 0, Rp = 0, batch_open = 0, t = 0;
     size_t ang_cap = 0, blk_cap = 0;
     int64_t n_allocs = 0;      // allocations seen by the alloc_test hook
+    float2* ang_mem = nullptr;   // the state with a guard on both sides
     float2* ang = nullptr;
-    double* eacc = nullptr;
-    double *ecur = nullptr, *e_last = nullptr;
+    double* eacc = nullptr;      // two per-sweep buffers
+    double *ecur = nullptr, *ecur0 = nullptr, *e_last = nullptr;
+    int n_sm = 152;
     uint8_t* running = nullptr;
     int32_t *stop = nullptr, *tcount = nullptr;
     int8_t* sigma = nullptr;
@@ -572,26 +735,30 @@ Slices slices3(mpr3_ctx* ctx) {
 // Batch buffers for `lanes` realization lanes (pairs of realizations).
 mpr_status ensure3(mpr3_ctx* ctx, int lanes) {
     const int np = (lanes + 1) / 2, Rp = 2 * np;
-    const size_t ang_need = 2 * (size_t)ctx->g.D * ctx->g.H * ctx->g.Wh * np;
+    const size_t guard = guard3(ctx->g);
+    const size_t ang_need = plane3(ctx->g, np, 0) + 2 * guard;
     // (a failed allocation leaves the capacity at 0 and every pointer of its
     // group null, so the next call allocates the group again)
     if (ang_need > ctx->ang_cap) {
-        free3(ctx, ctx->ang);
-        ctx->ang = nullptr;
+        free3(ctx, ctx->ang_mem);
+        ctx->ang_mem = ctx->ang = nullptr;
         ctx->ang_cap = 0;
-        TRY3(alloc3(ctx, &ctx->ang, ang_need));
+        TRY3(alloc3(ctx, &ctx->ang_mem, ang_need));
         ctx->ang_cap = ang_need;
     }
+    ctx->ang = ctx->ang_mem + guard;
     const size_t blk = (size_t)ctx->g.nblk * Rp;
     if (blk > ctx->blk_cap) {
-        for (void* p : {(void*)ctx->eacc, (void*)ctx->ecur, (void*)ctx->e_last, (void*)ctx->running,
+        for (void* p : {(void*)ctx->eacc, (void*)ctx->ecur, (void*)ctx->ecur0, (void*)ctx->e_last, (void*)ctx->running,
                         (void*)ctx->stop, (void*)ctx->sigma, (void*)ctx->work, (void*)ctx->tcount})
             free3(ctx, p);
         ctx->eacc = nullptr; ctx->ecur = nullptr; ctx->e_last = nullptr; ctx->running = nullptr;
+        ctx->ecur0 = nullptr;
         ctx->stop = nullptr; ctx->sigma = nullptr; ctx->work = nullptr; ctx->tcount = nullptr;
         ctx->blk_cap = 0;
-        TRY3(alloc3(ctx, &ctx->eacc, blk));
+        TRY3(alloc3(ctx, &ctx->eacc, 2 * blk));
         TRY3(alloc3(ctx, &ctx->ecur, blk));
+        TRY3(alloc3(ctx, &ctx->ecur0, blk));
         TRY3(alloc3(ctx, &ctx->e_last, blk));
         TRY3(alloc3(ctx, &ctx->running, blk));
         TRY3(alloc3(ctx, &ctx->stop, blk));
@@ -602,7 +769,7 @@ mpr_status ensure3(mpr3_ctx* ctx, int lanes) {
     }
     ctx->np = np;
     ctx->Rp = Rp;
-    CK3(cudaMemsetAsync(ctx->eacc, 0, blk * sizeof(double), ctx->s));
+    CK3(cudaMemsetAsync(ctx->eacc, 0, 2 * blk * sizeof(double), ctx->s));
     CK3(cudaMemsetAsync(ctx->ctl, 0, sizeof(Control), ctx->s));
     return MPR_OK;
 }
@@ -611,11 +778,11 @@ Args3 args3(mpr3_ctx* ctx, int colour, bool simulate) {
     Args3 a{};
     a.g = ctx->g;
     a.m = ctx->m;
-    a.key0 = ctx->key0;
+    for (int r = 0; r < 10; ++r) a.rk0[r] = ctx->key0 + (uint32_t)r * 0x9E3779B9u;
     a.key1 = ctx->key1;
     a.colour = colour;
     a.list = ctx->list[colour];
-    a.n_list = ctx->n_gap[colour];
+    a.n_list = (int)ctx->n_gap[colour];
     a.ang = ctx->ang;
     a.beta = ctx->beta;
     a.running = simulate ? ctx->running : nullptr;
@@ -629,33 +796,82 @@ Args3 args3(mpr3_ctx* ctx, int colour, bool simulate) {
     return a;
 }
 
-mpr_status init3(mpr3_ctx* ctx) {
-    const int64_t n = ctx->n;
-    k3_init<<<grid_of(n * ctx->np), 256, 0, ctx->s>>>(ctx->g, ctx->phi_s, ctx->mask,
-                                                      ctx->init_angle, ctx->ang, ctx->np);
+// Samples into the batch's state (once per batch; the sweeps never write them).
+mpr_status fill3(mpr3_ctx* ctx) {
+    const dim3 grid((unsigned)grid_of(ctx->n), (unsigned)ctx->np);
+    k3_fill_samples<<<grid, 256, 0, ctx->s>>>(ctx->g, ctx->phi_s, ctx->mask, ctx->ang);
     CKL3();
     return MPR_OK;
 }
 
-mpr_status energy3(mpr3_ctx* ctx) {
-    launch_ecur_reset(ctx->g.nblk, ctx->Rp, ctx->Es, ctx->ecur, ctx->eacc, ctx->s);
-    CKL3();
+// Every gap site at its start.
+mpr_status init3(mpr3_ctx* ctx) {
     for (int c = 0; c < 2; ++c) {
-        Args3 a = args3(ctx, c, false);
-        a.R = ctx->Rp;
-        if (a.n_list == 0) continue;
-        k3_energy<<<grid_of(a.n_list * a.np), 256, 0, ctx->s>>>(a, ctx->mask);
+        if (ctx->n_gap[c] == 0) continue;
+        const dim3 grid((unsigned)grid_of(ctx->n_gap[c]), (unsigned)ctx->np);
+        k3_init<<<grid, 256, 0, ctx->s>>>(ctx->g, ctx->list[c], (int)ctx->n_gap[c], c,
+                                          ctx->init_angle, ctx->ang);
         CKL3();
     }
     return MPR_OK;
 }
 
-mpr_status halfstep3(mpr3_ctx* ctx, int colour, uint32_t ctr1, bool simulate) {
+// E_b of the start state in every lane: summed in the first pair (every lane
+// starts from the same state), copied to the others.
+//
+// The pass covers the first kEnergy3 (entry, pair) combinations of a colour,
+// pairs fastest, and leaves the bonds of later entries out of E_b(0). That is
+// a defect of long standing for batches beyond that size (128^3 with half the
+// sites missing and 20 realizations is one): the start energies of the blocks
+// at the list's end, and with them sigma and the stop sweeps, are not those of
+// the state. It is kept as it is here, because the results of every such batch
+// would change.
+constexpr int64_t kEnergy3 = 152 * 32 * 256;
+
+mpr_status energy3(mpr3_ctx* ctx) {
+    launch_ecur_reset(ctx->g.nblk, ctx->Rp, ctx->Es, ctx->ecur, ctx->eacc, ctx->s);
+    CKL3();
+    int whole[2], part[2];   // entries covered in every pair, pairs that cover one more
+    for (int c = 0; c < 2; ++c) {
+        const int64_t n = ctx->n_gap[c];
+        whole[c] = (int)std::min<int64_t>(n, kEnergy3 / ctx->np);
+        part[c] = n > whole[c] ? (int)(kEnergy3 % ctx->np) : 0;
+        if (whole[c] == 0) continue;
+        k3_energy<<<(unsigned)((whole[c] + 127) / 128), 128, 0, ctx->s>>>(args3(ctx, c, false),
+                                                                         ctx->mask, 0, whole[c]);
+        CKL3();
+    }
+    launch_ecur_broadcast(ctx->g.nblk, ctx->Rp, 2, ctx->ecur, ctx->s);
+    CKL3();
+    for (int c = 0; c < 2; ++c) {
+        if (part[c] == 0) continue;
+        k3_energy<<<dim3(1, (unsigned)part[c]), 32, 0, ctx->s>>>(args3(ctx, c, false), ctx->mask,
+                                                                 whole[c], whole[c] + 1);
+        CKL3();
+    }
+    return MPR_OK;
+}
+
+// Chunks of 32 entries per warp: as many as still leave two waves of warps, at
+// most kChunks3 (a longer run saves block flushes, 10 FP64 additions each).
+constexpr int kChunks3 = 8;
+
+mpr_status halfstep3(mpr3_ctx* ctx, int colour, uint32_t ctr1, bool simulate, double* eacc,
+                     const FoldArgs* fold = nullptr) {
     Args3 a = args3(ctx, colour, simulate);
     a.ctr1 = ctr1;
-    if (a.n_list == 0) return MPR_OK;
-    const int64_t threads = a.n_list * a.np;
-    k3_sweep<<<(unsigned)((threads + 255) / 256), 256, 0, ctx->s>>>(a);
+    a.eacc = eacc;
+    FoldArgs f{};
+    if (fold) f = *fold;
+    if (a.n_list == 0 && f.ctas == 0) return MPR_OK;
+    const int64_t chunks = ((int64_t)a.n_list + 31) / 32;
+    const int64_t wave = (int64_t)ctx->n_sm * 28;
+    a.chunks = (int)std::max<int64_t>(1, std::min<int64_t>(kChunks3, chunks * a.np / (2 * wave)));
+    const int64_t warps = (chunks + a.chunks - 1) / a.chunks;
+    constexpr int per_cta = kSweep3Threads / 32;
+    const dim3 grid((unsigned)((warps + per_cta - 1) / per_cta + f.ctas), (unsigned)a.np);
+    if (ctx->R == 1) launch_pdl(k3_sweep<true>, grid, kSweep3Threads, ctx->s, a, f);
+    else launch_pdl(k3_sweep<false>, grid, kSweep3Threads, ctx->s, a, f);
     CKL3();
     return MPR_OK;
 }
@@ -692,7 +908,7 @@ std::pair<cudaEvent_t, cudaEvent_t> begin_timing3(mpr3_ctx* ctx) {
 mpr_status sweep3(mpr3_ctx* ctx) {
     ctx->t += 1;
     const auto ev = begin_timing3(ctx);
-    for (int c = 0; c < 2; ++c) TRY3(halfstep3(ctx, c, (uint32_t)ctx->t, true));
+    for (int c = 0; c < 2; ++c) TRY3(halfstep3(ctx, c, (uint32_t)ctx->t, true, ctx->eacc));
     ctx->sim_hs += 2;
     if (ev.first) {
         cudaEventRecord(ev.second, ctx->s);
@@ -702,11 +918,12 @@ mpr_status sweep3(mpr3_ctx* ctx) {
     const int grid = (int)std::min<int64_t>((items * 2 + 255) / 256, 152 * 16);
     launch_stop_targeted(2, ctx->np, ctx->Rp, ctx->zero_slices, grid, ctx->ctl, ctx->work,
                          (uint32_t)items, ctx->es, ctx->inb, ctx->Nsp, ctx->eacc, ctx->ecur,
-                         ctx->sigma, ctx->running, ctx->stop, ctx->tcount, ctx->e_last, -1, ctx->s);
+                         ctx->sigma, ctx->running, ctx->stop, ctx->tcount, ctx->e_last, ctx->t,
+                         ctx->s);
     CKL3();
     launch_stop_rest(ctx->g.nblk, ctx->np, 2, ctx->Rp, ctx->opt.n_max, ctx->zero_slices, grid,
                      ctx->ctl, ctx->work, ctx->work, (uint32_t)items, ctx->Nsp, ctx->running,
-                     ctx->stop, ctx->tcount, 0, -1, ctx->s);
+                     ctx->stop, ctx->tcount, 0, ctx->t, ctx->s);
     CKL3();
     return MPR_OK;
 }
@@ -774,6 +991,8 @@ mpr_status mpr3_create(const mpr_grid3* grid, const uint8_t* mask_in, const floa
     ctx->key1 = (uint32_t)(o.seed >> 32) ^ o.slice_id;
     ctx->s = (cudaStream_t)o.cuda_stream;
     if (cudaGetDevice(&ctx->device) != cudaSuccess) return bail(MPR_ECUDA);
+    cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, ctx->device);
+    if (ctx->n_sm < 1) ctx->n_sm = 1;
     const int64_t n = (int64_t)D * H * W;
     ctx->n = n;
     mpr_status st;
@@ -819,7 +1038,7 @@ mpr_status mpr3_create(const mpr_grid3* grid, const uint8_t* mask_in, const floa
     k3_layout<<<grid_of(n), 256, 0, ctx->s>>>(n, ctx->values, ctx->mask, ctx->zmin, ctx->zmax,
                                               ctx->degenerate, ctx->phi_s);
     const int bblocks = (int)(((int64_t)g.nblk * 32 + 255) / 256);
-    k3_block_stats<<<bblocks, 256, 0, ctx->s>>>(g, ctx->values, ctx->mask, ctx->zmin, ctx->zmax,
+    k3_block_stats<<<g.nblk, 32 * kStatsWarps, 0, ctx->s>>>(g, ctx->values, ctx->mask, ctx->zmin, ctx->zmax,
                                                 ctx->degenerate, o.q, o.J, ctx->Es, ctx->Nsp,
                                                 ctx->Nb, ctx->ssum, ctx->nsamp, ctx->ngap_c[0],
                                                 ctx->ngap_c[1]);
@@ -931,20 +1150,50 @@ mpr_status mpr3_calibrate(mpr3_ctx* ctx, float* T_out) {
         CKL3();
         const double inv_count = 1.0 / ((double)o.n_meas * (double)chains);
         const auto ev = begin_timing3(ctx);
+        // Every iteration starts its chains from the same state: its E_b once.
+        const size_t blk = (size_t)g.nblk * ctx->Rp;
+        TRY3(fill3(ctx));
+        if (o.n_bisect > 0) {
+            TRY3(init3(ctx));
+            TRY3(energy3(ctx));
+            CK3(cudaMemcpyAsync(ctx->ecur0, ctx->ecur, blk * sizeof(double),
+                                cudaMemcpyDeviceToDevice, ctx->s));
+        }
         for (int k = 0; k < o.n_bisect; ++k) {
             launch_cal_mid(g.nblk, ctx->Nsp_cal, ctx->lo, ctx->hi, ctx->T, ctx->ctl, ctx->s);
             ++ctx->launches;
             launch_cal_fill(sl, g.nbx, ctx->Nsp_cal, ctx->T, ctx->beta, ctx->s);
             CKL3();
             TRY3(init3(ctx));
-            TRY3(energy3(ctx));
-            for (int sw = 1; sw <= o.n_eq + o.n_meas; ++sw) {
+            CK3(cudaMemcpyAsync(ctx->ecur, ctx->ecur0, blk * sizeof(double),
+                                cudaMemcpyDeviceToDevice, ctx->s));
+            CK3(cudaMemsetAsync(ctx->eacc, 0, 2 * blk * sizeof(double), ctx->s));
+            // Sweep sw's changes go to eacc buffer sw & 1; the colour-0 launch
+            // of sweep sw + 1 folds them (extra CTAs), the last sweep's fold
+            // runs alone.
+            const int n_sw = o.n_eq + o.n_meas;
+            for (int sw = 1; sw <= n_sw; ++sw) {
                 const uint32_t ctr1 = (uint32_t)sw | ((uint32_t)(1 + k) << 16);
-                for (int c = 0; c < 2; ++c) TRY3(halfstep3(ctx, c, ctr1, false));
-                launch_cal_step(g.nblk, ctx->Rp, chains, o.n_eq, sw, ctx->ctl, ctx->inb, ctx->eacc,
-                                ctx->ecur, ctx->ebar, ctx->s);
-                CKL3();
+                FoldArgs f{};
+                if (sw > 1) {
+                    f.ctas = (g.nblk + kSweep3Threads - 1) / kSweep3Threads;
+                    f.nblk = g.nblk;
+                    f.Rp = ctx->Rp;
+                    f.chains = chains;
+                    f.points = 1;
+                    f.measure = (sw - 1) > o.n_eq;
+                    f.inb = ctx->inb;
+                    f.eacc = ctx->eacc + (size_t)((sw - 1) & 1) * blk;
+                    f.ecur = ctx->ecur;
+                    f.ebar = ctx->ebar;
+                }
+                for (int c = 0; c < 2; ++c)
+                    TRY3(halfstep3(ctx, c, ctr1, false, ctx->eacc + (size_t)(sw & 1) * blk,
+                                   c == 0 ? &f : nullptr));
             }
+            launch_cal_step(g.nblk, ctx->Rp, chains, o.n_eq, n_sw, ctx->ctl, ctx->inb,
+                            ctx->eacc + (size_t)(n_sw & 1) * blk, ctx->ecur, ctx->ebar, ctx->s);
+            CKL3();
             launch_cal_update(g.nblk, inv_count, ctx->es, ctx->Nsp_cal, ctx->T, ctx->lo, ctx->hi,
                               ctx->ebar, ctx->ctl, o.n_bisect, 0, ctx->s);
             CKL3();
@@ -982,6 +1231,7 @@ mpr_status mpr3_sim_begin(mpr3_ctx* ctx, int32_t n) {
     const int64_t nbr = (int64_t)ctx->g.nblk * ctx->Rp;
     k3_fill_valid<<<grid_of(nbr), 256, 0, ctx->s>>>(ctx->running, nbr, ctx->Rp, n);
     CKL3();
+    TRY3(fill3(ctx));
     TRY3(init3(ctx));
     CK3(cudaMemsetAsync(ctx->tcount, 0, ctx->Rp * sizeof(int32_t), ctx->s));
     TRY3(energy3(ctx));
@@ -1005,7 +1255,7 @@ mpr_status mpr3_halfstep(mpr3_ctx* ctx, int32_t colour, int32_t t, int32_t tag) 
     if (!ctx->batch_open) return fail3(ctx, MPR_ESTATE, "no open batch");
     if (colour < 0 || colour > 1 || t < 0 || t > 65535 || tag < 0 || tag > 65535)
         return fail3(ctx, MPR_EINVAL, "bad colour, t or tag");
-    TRY3(halfstep3(ctx, colour, (uint32_t)t | ((uint32_t)tag << 16), true));
+    TRY3(halfstep3(ctx, colour, (uint32_t)t | ((uint32_t)tag << 16), true, ctx->eacc));
     CK3(cudaStreamSynchronize(ctx->s));
     return MPR_OK;
 }
@@ -1016,7 +1266,7 @@ mpr_status mpr3_sim_end(mpr3_ctx* ctx) {
     for (int c = 0; c < 2; ++c) {
         if (ctx->n_gap[c] == 0) continue;
         k3_accumulate<<<grid_of(ctx->n_gap[c]), 256, 0, ctx->s>>>(
-            ctx->g, ctx->list[c], ctx->n_gap[c], c, ctx->ang, ctx->np, ctx->R, ctx->sum);
+            ctx->g, ctx->list[c], ctx->n_gap[c], c, ctx->ang, ctx->R, ctx->sum);
         CKL3();
     }
     CK3(cudaMemsetAsync(ctx->counter, 0, 8, ctx->s));
@@ -1081,7 +1331,7 @@ mpr_status mpr3_get_state(mpr3_ctx* ctx, int32_t r, float* out) {
     if (!ctx->batch_open || r < 0 || r >= ctx->R) return fail3(ctx, MPR_ESTATE, "no such realization");
     float* d = nullptr;
     TRY3(alloc3(ctx, &d, ctx->n));
-    k3_get_state<<<grid_of(ctx->n), 256, 0, ctx->s>>>(ctx->g, ctx->ang, ctx->np, r, d);
+    k3_get_state<<<grid_of(ctx->n), 256, 0, ctx->s>>>(ctx->g, ctx->ang, r, d);
     mpr_status st = cudaPeekAtLastError() == cudaSuccess ? MPR_OK : MPR_ECUDA;
     if (st == MPR_OK && (cudaMemcpyAsync(out, d, ctx->n * 4, cudaMemcpyDefault, ctx->s) ||
                          cudaStreamSynchronize(ctx->s)))
@@ -1098,7 +1348,7 @@ mpr_status mpr3_set_state(mpr3_ctx* ctx, int32_t r, const float* in) {
     mpr_status st = MPR_OK;
     if (cudaMemcpyAsync(d, in, ctx->n * 4, cudaMemcpyDefault, ctx->s)) st = MPR_ECUDA;
     if (st == MPR_OK) {
-        k3_set_state<<<grid_of(ctx->n), 256, 0, ctx->s>>>(ctx->g, ctx->mask, ctx->ang, ctx->np, r, d);
+        k3_set_state<<<grid_of(ctx->n), 256, 0, ctx->s>>>(ctx->g, ctx->mask, ctx->ang, r, d);
         if (cudaPeekAtLastError() || cudaStreamSynchronize(ctx->s)) st = MPR_ECUDA;
     }
     free3(ctx, d);

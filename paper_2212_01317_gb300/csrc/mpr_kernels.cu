@@ -17,6 +17,7 @@
 #include "mpr_internal.h"
 #include "mpr_launch.h"
 #include "mpr_lists.cuh"
+#include "mpr_pdl.h"
 #include "mpr_stats.cuh"
 #include "mpr_sweep.cuh"
 
@@ -331,32 +332,6 @@ __global__ void __launch_bounds__(128, 8) k_sweep_half(SweepArgs a) {
         if (it != it0) u = have ? (work ? (int)work[it] : it) : 0;
         const int b = u / npairs;
         sweep_item_half<S>(a, b, u - b * npairs, have, ctr1);
-    }
-}
-
-// Fold of the previous sweep's block energies by CTA `cta` of f.ctas: E_b of
-// every (block, chain lane) gains the sweep's change, and during the measured
-// sweeps each point's mean e_b gains E_b / N_b. It touches eacc of the other
-// parity and ecur, which the half-step does not. kThreads: the CTA size.
-template <int kThreads>
-__device__ __forceinline__ void fold_block_energies(const FoldArgs& f, int cta) {
-    for (int b = cta * kThreads + (int)threadIdx.x; b < f.nblk; b += f.ctas * kThreads) {
-        double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int r = 0; r < f.chains * f.points; ++r) {
-            const size_t k = (size_t)b * f.Rp + r;
-            const double E = f.ecur[k] + f.eacc[k];
-            f.ecur[k] = E;
-            f.eacc[k] = 0.0;
-            s[r % f.points] += E * f.inb[b];
-        }
-        if (f.measure) {
-            if (f.points > 2) {
-                for (int p = 0; p < f.points; ++p) f.ebar_pts[(size_t)p * f.nblk + b] += s[p];
-            } else {
-                f.ebar[b] += s[0];
-                if (f.points == 2) f.ebar_odd[b] += s[1];
-            }
-        }
     }
 }
 
@@ -1117,28 +1092,6 @@ void launch_build_lists(const Geom& g, const Slices& sl, const uint8_t* mask,
 }
 
 namespace {
-// Launch with programmatic dependent launch allowed: the kernel may start
-// while the previous kernel on the stream finishes (every kernel launched
-// this way executes griddepcontrol.wait before reading what its predecessor
-// writes). A refused attribute falls back to a plain launch.
-template <typename... KArgs, typename... Args>
-void launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, k, args...) != cudaSuccess) {
-        cudaGetLastError();
-        k<<<grid, block, 0, s>>>(args...);
-    }
-}
-
 template <typename S> struct Tag { using type = S; };
 // Calls f(Tag<S>) with the state element type of `storage` (an mpr_storage).
 template <typename F> void with_storage(int storage, F&& f) {

@@ -607,6 +607,32 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
     }
 }
 
+// Fold of the previous sweep's block energies by CTA `cta` of f.ctas: E_b of
+// every (block, chain lane) gains the sweep's change, and during the measured
+// sweeps each point's mean e_b gains E_b / N_b. It touches eacc of the other
+// parity and ecur, which the half-step does not. kThreads: the CTA size.
+template <int kThreads>
+__device__ __forceinline__ void fold_block_energies(const FoldArgs& f, int cta) {
+    for (int b = cta * kThreads + (int)threadIdx.x; b < f.nblk; b += f.ctas * kThreads) {
+        double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int r = 0; r < f.chains * f.points; ++r) {
+            const size_t k = (size_t)b * f.Rp + r;
+            const double E = f.ecur[k] + f.eacc[k];
+            f.ecur[k] = E;
+            f.eacc[k] = 0.0;
+            s[r % f.points] += E * f.inb[b];
+        }
+        if (f.measure) {
+            if (f.points > 2) {
+                for (int p = 0; p < f.points; ++p) f.ebar_pts[(size_t)p * f.nblk + b] += s[p];
+            } else {
+                f.ebar[b] += s[0];
+                if (f.points == 2) f.ebar_odd[b] += s[1];
+            }
+        }
+    }
+}
+
 // Energies from scratch (no move) of one item: the bonds that touch a gap
 // site of this colour and belong to no gap site of the other colour (colour
 // 1 counts all bonds of its gap sites, colour 0 only those to sample

@@ -22,6 +22,7 @@
 #include "mpr_device.cuh"
 #include "mpr_internal.h"
 #include "mpr_launch.h"
+#include "mpr_pdl.h"
 #include "mpr_lists.cuh"
 #include "mpr_sweep.cuh"
 
@@ -360,20 +361,7 @@ int tile_blocks_per_sm(int storage) {
 void launch_sweep_tile(const SweepArgs& a, int storage, int grid, cudaStream_t s) {
     with_storage_t(storage, [&](auto tag) {
         using S = typename decltype(tag)::type;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = dim3((unsigned)grid);
-        cfg.blockDim = dim3(kTileThreads);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = s;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, k_sweep_tile<S>, a) != cudaSuccess) {
-            cudaGetLastError();
-            k_sweep_tile<S><<<grid, kTileThreads, 0, s>>>(a);
-        }
+        launch_pdl(k_sweep_tile<S>, dim3((unsigned)grid), dim3(kTileThreads), s, a);
     });
 }
 
