@@ -215,6 +215,22 @@ struct FoldArgs {
     double* ebar_pts;         // [points][nblk] (points > 2: lane r adds to point r mod points)
 };
 
+// One calibration iteration of a small field, a cluster per realization pair
+// (mpr_calcluster.cu): at most kCalClusterSites gap sites per colour.
+constexpr int kCalClusterSites = 8192;
+struct CalClusterArgs {
+    SweepArgs sw;              // beta / beta_odd / beta_pts, n_pts, ang, ctl, R, Rp, ...
+    const uint4* list[2];
+    int n_list[2];
+    const float* init_angle;   // [nblk]
+    int random_init;
+    const double* E0;          // [nblk][Rp] E_b of the start
+    const double* inb;         // [nblk] 1 / N_b
+    int n_sweeps, n_meas;      // the last n_meas of n_sweeps are measured
+    int points;
+    double *ebar, *ebar_odd, *ebar_pts;   // as FoldArgs
+};
+
 // Grid-wide barrier state of a cooperative launch (zeroed before each launch).
 struct GridBarrier {
     unsigned int arrive;   // CTAs arrived at the current barrier

@@ -159,6 +159,11 @@ void launch_tile_lists(const Geom& g, const Tiles& tl, const int32_t* of_block,
 int tile_blocks_per_sm(int storage);
 void launch_sweep_tile(const SweepArgs& a, int storage, int grid, cudaStream_t s);
 
+// The calibration iteration of a small field as one launch: clusters that fit
+// the GPU at once (0: not available), and the launch.
+int cal_cluster_max_active();
+cudaError_t launch_cal_cluster(const CalClusterArgs& a, cudaStream_t s);
+
 int cal_persistent_blocks_per_sm(int G);
 cudaError_t launch_cal_persistent(const CalPersistArgs& a, int G, int grid, cudaStream_t s);
 

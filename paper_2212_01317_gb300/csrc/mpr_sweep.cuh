@@ -97,16 +97,14 @@ template <> struct Store<__nv_bfloat16> {
 // Site update with the state's rounding applied: the proposal is rounded
 // before its energy is taken, so the Metropolis test judges the angle that
 // is stored; the reflected angle is rounded too, and for the 16-bit forms
-// dE is the exact change from the old to the stored final angle. Sn, C: the
-// local field. The roundings are spelled out (see bond_change).
+// dE is the exact change from the old to the stored final angle. (co, so):
+// cos, sin of q phi; php, (cp, sp): the rounded proposal and its cos, sin;
+// C, Sn: the local field. The roundings are spelled out (see bond_change).
 template <typename S>
-__device__ __forceinline__ SiteNew site_update(float phi, float C, float Sn, float u0, float u1,
-                                               float beta, const Model& m) {
+__device__ __forceinline__ SiteNew site_move(float phi, float co, float so, float php, float cp,
+                                             float sp, float C, float Sn, float u1, float beta,
+                                             const Model& m) {
     SiteNew n;
-    float co, so, cp, sp;
-    __sincosf(m.q * phi, &so, &co);
-    const float php = Store<S>::round(kTwoPi * u0);
-    __sincosf(m.q * php, &sp, &cp);
     const float e0 = __fmaf_rn(Sn, so, __fmul_rn(C, co));
     const float e1 = __fmaf_rn(Sn, sp, __fmul_rn(C, cp));
     const float dE = __fmul_rn(m.J, __fsub_rn(e0, e1));
@@ -132,6 +130,16 @@ __device__ __forceinline__ SiteNew site_update(float phi, float C, float Sn, flo
     return n;
 }
 
+template <typename S>
+__device__ __forceinline__ SiteNew site_update(float phi, float C, float Sn, float u0, float u1,
+                                               float beta, const Model& m) {
+    float co, so, cp, sp;
+    __sincosf(m.q * phi, &so, &co);
+    const float php = Store<S>::round(kTwoPi * u0);
+    __sincosf(m.q * php, &sp, &cp);
+    return site_move<S>(phi, co, so, php, cp, sp, C, Sn, u1, beta, m);
+}
+
 // site_update of a site in both realizations of a pair, with the same roundings
 // (bit for bit): what is not a hardware function or a choice is packed two-wide
 // FP32 arithmetic, one instruction for both realizations. The half-step is
@@ -148,14 +156,11 @@ __device__ __forceinline__ SiteNew site_update(float phi, float C, float Sn, flo
 // BF16 sweeps); loads one entry ahead into registers, bulk prefetches of the
 // next unit's rows into L2, and 7, 9 or 10 CTAs per SM were slower too.
 template <typename S>
-__device__ __forceinline__ PairNew pair_update(float2 phi, float2 C, float2 Sn, float2 u0,
-                                               float2 u1, float2 beta, const Model& m) {
+__device__ __forceinline__ PairNew pair_move(float2 phi, float2 co, float2 so, float2 php,
+                                             float2 cp, float2 sp, float2 C, float2 Sn, float2 u1,
+                                             float2 beta, const Model& m) {
     PairNew n;
     const float2 q2 = both(m.q), J2 = both(m.J);
-    float2 co, so, cp, sp;
-    sincos_2(__fmul2_rn(q2, phi), so, co);
-    const float2 php = Store<S>::round2(__fmul2_rn(both(kTwoPi), u0));
-    sincos_2(__fmul2_rn(q2, php), sp, cp);
     const float2 e0 = __ffma2_rn(Sn, so, __fmul2_rn(C, co));
     const float2 e1 = __ffma2_rn(Sn, sp, __fmul2_rn(C, cp));
     n.dE = __fmul2_rn(J2, __ffma2_rn(e1, both(-1.0f), e0));
@@ -180,6 +185,17 @@ __device__ __forceinline__ PairNew pair_update(float2 phi, float2 C, float2 Sn, 
         n.dE = __fmul2_rn(J2, __ffma2_rn(e2, both(-1.0f), e0));
     }
     return n;
+}
+
+template <typename S>
+__device__ __forceinline__ PairNew pair_update(float2 phi, float2 C, float2 Sn, float2 u0,
+                                               float2 u1, float2 beta, const Model& m) {
+    const float2 q2 = both(m.q);
+    float2 co, so, cp, sp;
+    sincos_2(__fmul2_rn(q2, phi), so, co);
+    const float2 php = Store<S>::round2(__fmul2_rn(both(kTwoPi), u0));
+    sincos_2(__fmul2_rn(q2, php), sp, cp);
+    return pair_move<S>(phi, co, so, php, cp, sp, C, Sn, u1, beta, m);
 }
 
 // A block's change in one half-step: the FP32 warp sum of the unit's moves
