@@ -1042,8 +1042,7 @@ mpr_status mpr3_create(const mpr_grid3* grid, const uint8_t* mask_in, const floa
                                                 ctx->degenerate, o.q, o.J, ctx->Es, ctx->Nsp,
                                                 ctx->Nb, ctx->ssum, ctx->nsamp, ctx->ngap_c[0],
                                                 ctx->ngap_c[1]);
-    launch_scan(ctx->ngap_c[0], g.nblk, ctx->start[0], ctx->s);
-    launch_scan(ctx->ngap_c[1], g.nblk, ctx->start[1], ctx->s);
+    launch_scan(ctx->ngap_c[0], ctx->ngap_c[1], g.nblk, ctx->start[0], ctx->start[1], ctx->s);
     std::vector<int32_t> s0(g.nblk + 1), s1(g.nblk + 1), nsp(g.nblk), nsm(g.nblk), ng0(g.nblk),
         ng1(g.nblk), nbv(g.nblk);
     std::vector<double> ssum(g.nblk), esv(g.nblk);

@@ -448,11 +448,10 @@ mpr_status ensure_tiles(mpr_ctx* ctx) {
     }
     launch_stage_table(g, ctx->mask, ctx->dang, ctx->stab, ctx->s);
     launch_tile_count(g, t, ctx->d_of_block, ctx->mask, cnt[0], cnt[1], ctx->s);
-    launch_scan(cnt[0], t.n, ctx->tstart[0], ctx->s);
-    launch_scan(cnt[1], t.n, ctx->tstart[1], ctx->s);
+    launch_scan(cnt[0], cnt[1], t.n, ctx->tstart[0], ctx->tstart[1], ctx->s);
     launch_tile_lists(g, t, ctx->d_of_block, ctx->mask, ctx->tstart[0], ctx->tstart[1],
                       ctx->tlist[0], ctx->tlist[1], ctx->s);
-    ctx->launches += 5;
+    ctx->launches += 4;
     CKL();
     dfree(ctx, cnt[0]);
     dfree(ctx, cnt[1]);
@@ -1254,23 +1253,6 @@ void mpr_destroy(mpr_ctx* ctx) {
 
 namespace {
 
-// Canvas mask: 1 gap / 0 sample inside every slice's field (any nonzero
-// input is a gap), 2 everywhere else.
-__global__ void k_mask_normalize(Geom g, Slices sl, uint8_t* __restrict__ mask) {
-    const int64_t n = (int64_t)g.H * g.W;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int y = (int)(i / g.W), x = (int)(i % g.W);
-        const int s = sl.of_block[(y / g.lb) * g.nbx + x / g.lb];
-        bool inside = false;
-        if (s >= 0) {
-            const int4 rc = sl.rect[s];
-            inside = y < rc.x + rc.z && x < rc.y + rc.w;
-        }
-        mask[i] = inside ? (mask[i] != 0 ? MASK_GAP : 0) : MASK_ABSENT;
-    }
-}
-
 struct SliceDesc {
     int y0, x0, H, W;
 };
@@ -1448,116 +1430,69 @@ mpr_status create_impl(const mpr_options* opt_in, int H, int W, int lb,
         const mpr_status us = upload(ctx);
         if (us != MPR_OK) return bail(us);
     }
-    k_mask_normalize<<<(int)std::min<int64_t>((n + 255) / 256, 152 * 16), 256, 0, ctx->s>>>(
-        g, ctx->sl, ctx->mask);
-    ++ctx->launches;
-    // z_min / z_max over the samples of every slice.
+    // Canvas mask and sample ranges, Eq. 2 statistics and sample angles, per-block
+    // constants, list sizes: one chain of kernels, read back once.
+    SliceTotals* d_tot = nullptr;
+    ST(dalloc(ctx, &d_tot, ns));
     {
+        // (min starts from the largest integer, max from 0)
         std::vector<uint32_t> mm(2 * (size_t)ns);
-        for (int k = 0; k < ns; ++k) { mm[2 * k] = 0xffffffffu; mm[2 * k + 1] = 0u; }
+        for (int k = 0; k < ns; ++k) mm[2 * k] = 0xffffffffu;
         if (cudaMemcpyAsync(ctx->mm, mm.data(), mm.size() * 4, cudaMemcpyHostToDevice, ctx->s) !=
             cudaSuccess)
             return bail(MPR_ECUDA);
-        launch_minmax(g, ctx->d_of_block, ctx->values, ctx->mask, ctx->mm, ctx->s);
-        ++ctx->launches;
-        if (cudaMemcpyAsync(mm.data(), ctx->mm, mm.size() * 4, cudaMemcpyDeviceToHost, ctx->s) !=
-                cudaSuccess ||
-            cudaStreamSynchronize(ctx->s) != cudaSuccess)
-            return bail(MPR_ECUDA);
-        ctx->h_zmin.assign(ns, 0.0);
-        ctx->h_zmax.assign(ns, 0.0);
-        ctx->h_degen.assign(ns, 1);
-        for (int k = 0; k < ns; ++k) {
-            if (mm[2 * k] == 0xffffffffu) continue;   // no sample in the slice
-            ctx->h_zmin[k] = (double)ord2f(mm[2 * k]);
-            ctx->h_zmax[k] = (double)ord2f(mm[2 * k + 1]);
-            ctx->h_degen[k] = !(ctx->h_zmax[k] > ctx->h_zmin[k]);
-        }
-        ctx->zmin = ctx->h_zmin[0];
-        ctx->zmax = ctx->h_zmax[0];
-        ctx->degenerate = 1;     // every slice constant: nothing to calibrate
-        for (int k = 0; k < ns; ++k) ctx->degenerate &= ctx->h_degen[k];
-        if (cudaMemcpyAsync(ctx->d_zmin, ctx->h_zmin.data(), ns * 8, cudaMemcpyHostToDevice, ctx->s) ||
-            cudaMemcpyAsync(ctx->d_zmax, ctx->h_zmax.data(), ns * 8, cudaMemcpyHostToDevice, ctx->s) ||
-            cudaMemcpyAsync(ctx->d_degen, ctx->h_degen.data(), ns * 4, cudaMemcpyHostToDevice,
-                            ctx->s))
-            return bail(MPR_ECUDA);
     }
-    launch_layout(g, ctx->sl, ctx->values, ctx->mask, ctx->dang, ctx->s);
+    launch_prepare(g, ctx->sl, ctx->values, ctx->mask, ctx->mm, ctx->s);
+    launch_slice_range(ns, ctx->mm, ctx->d_zmin, ctx->d_zmax, ctx->d_degen, d_tot, ctx->s);
     launch_block_stats(g, ctx->sl, ctx->values, ctx->mask, ctx->opt.q, ctx->opt.J, ctx->Es,
                        ctx->Nsp, ctx->Nb, ctx->ssum, ctx->nsamp, ctx->ngap_c[0], ctx->ngap_c[1],
-                       ctx->s);
-    launch_scan(ctx->ngap_c[0], g.nblk, ctx->start[0], ctx->s);
-    launch_scan(ctx->ngap_c[1], g.nblk, ctx->start[1], ctx->s);
-    ctx->launches += 4;
-    if (cudaPeekAtLastError() != cudaSuccess) return bail(MPR_ECUDA);
-
-    // Host-side bookkeeping: list sizes, initial angles, sample-pair check.
-    std::vector<int32_t> s0(g.nblk + 1), s1(g.nblk + 1), nsp(g.nblk), nsm(g.nblk), ng0(g.nblk),
-        ng1(g.nblk), nbv(g.nblk);
-    std::vector<double> ssum(g.nblk), esv(g.nblk);
-    if (cudaMemcpyAsync(s0.data(), ctx->start[0], s0.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(s1.data(), ctx->start[1], s1.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(nsp.data(), ctx->Nsp, nsp.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(nsm.data(), ctx->nsamp, nsm.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(ng0.data(), ctx->ngap_c[0], ng0.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(ng1.data(), ctx->ngap_c[1], ng1.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(ssum.data(), ctx->ssum, ssum.size() * 8, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(esv.data(), ctx->Es, esv.size() * 8, cudaMemcpyDeviceToHost, ctx->s) ||
-        cudaMemcpyAsync(nbv.data(), ctx->Nb, nbv.size() * 4, cudaMemcpyDeviceToHost, ctx->s) ||
+                       ctx->dang, d_tot, ctx->s);
+    launch_block_finish(g.nblk, ctx->d_of_block, ctx->Es, ctx->Nsp, ctx->Nb, ctx->ssum, ctx->nsamp,
+                        ctx->ngap_c[0], ctx->ngap_c[1], d_tot, ctx->es, ctx->inb, ctx->ngap,
+                        ctx->Nsp_cal, ctx->init_angle, ctx->s);
+    launch_scan(ctx->ngap_c[0], ctx->ngap_c[1], g.nblk, ctx->start[0], ctx->start[1], ctx->s);
+    ctx->launches += 5;
+    std::vector<SliceTotals> tot(ns);
+    int32_t n_list[2] = {0, 0};
+    if (cudaPeekAtLastError() != cudaSuccess ||
+        cudaMemcpyAsync(tot.data(), d_tot, ns * sizeof(SliceTotals), cudaMemcpyDeviceToHost,
+                        ctx->s) ||
+        cudaMemcpyAsync(&n_list[0], ctx->start[0] + g.nblk, 4, cudaMemcpyDeviceToHost, ctx->s) ||
+        cudaMemcpyAsync(&n_list[1], ctx->start[1] + g.nblk, 4, cudaMemcpyDeviceToHost, ctx->s) ||
         cudaStreamSynchronize(ctx->s))
         return bail(MPR_ECUDA);
-    ctx->n_gap[0] = s0[g.nblk];
-    ctx->n_gap[1] = s1[g.nblk];
-    // Per slice: sample pairs (Eq. 2 needs one), gap sites, global sample mean.
-    std::vector<int64_t> pairs(ns, 0), samples(ns, 0);
-    std::vector<double> gsum(ns, 0.0);
+    dfree(ctx, d_tot);
+    ctx->device_bytes -= (int64_t)(ns * sizeof(SliceTotals));
+    ctx->n_gap[0] = n_list[0];
+    ctx->n_gap[1] = n_list[1];
     ctx->h_ngap.assign(ns, 0);
-    std::vector<float> init(g.nblk, 0.0f);
-    std::vector<int32_t> ng(g.nblk);
-    for (int b = 0; b < g.nblk; ++b) {
-        ng[b] = ng0[b] + ng1[b];
-        const int k = of_block[b];
-        if (k < 0) continue;
-        pairs[k] += nsp[b];
-        samples[k] += nsm[b];
-        gsum[k] += ssum[b];
-        ctx->h_ngap[k] += ng[b];
+    ctx->h_zmin.assign(ns, 0.0);
+    ctx->h_zmax.assign(ns, 0.0);
+    ctx->h_degen.assign(ns, 1);
+    ctx->degenerate = 1;     // every slice constant: nothing to calibrate
+    for (int k = 0; k < ns; ++k) {
+        ctx->h_ngap[k] = (int64_t)tot[k].gaps;
+        ctx->h_zmin[k] = tot[k].zmin;
+        ctx->h_zmax[k] = tot[k].zmax;
+        ctx->h_degen[k] = !(tot[k].zmax > tot[k].zmin);
+        ctx->degenerate &= ctx->h_degen[k];
+        // Eq. 2 needs a sample pair per slice that has gaps.
+        if (tot[k].pairs == 0 && tot[k].gaps > 0) return bail(MPR_ENOSAMPLES);
     }
-    for (int k = 0; k < ns; ++k)
-        if (pairs[k] == 0 && ctx->h_ngap[k] > 0) {
-            mpr_destroy(ctx);
-            return MPR_ENOSAMPLES;
-        }
-    for (int b = 0; b < g.nblk; ++b) {
-        const int k = of_block[b];
-        if (k < 0) continue;
-        const double gmean = samples[k] ? gsum[k] / (double)samples[k] : 0.0;
-        init[b] = (float)(nsm[b] > 0 ? ssum[b] / (double)nsm[b] : gmean);
-    }
-    std::vector<double> es_h(g.nblk), inb_h(g.nblk);
-    std::vector<int32_t> nsp_cal(g.nblk);
-    for (int b = 0; b < g.nblk; ++b) {
-        es_h[b] = nsp[b] > 0 ? esv[b] / (double)nsp[b] : 0.0;
-        inb_h[b] = nbv[b] > 0 ? 1.0 / (double)nbv[b] : 0.0;
-        nsp_cal[b] = ng[b] > 0 ? nsp[b] : 0;
-    }
+    ctx->zmin = ctx->h_zmin[0];
+    ctx->zmax = ctx->h_zmax[0];
     ST(dalloc(ctx, &ctx->list[0], ctx->n_gap[0]));
     ST(dalloc(ctx, &ctx->list[1], ctx->n_gap[1]));
-    if (cudaMemcpyAsync(ctx->init_angle, init.data(), g.nblk * 4, cudaMemcpyHostToDevice, ctx->s) ||
-        cudaMemcpyAsync(ctx->es, es_h.data(), g.nblk * 8, cudaMemcpyHostToDevice, ctx->s) ||
-        cudaMemcpyAsync(ctx->inb, inb_h.data(), g.nblk * 8, cudaMemcpyHostToDevice, ctx->s) ||
-        cudaMemcpyAsync(ctx->ngap, ng.data(), g.nblk * 4, cudaMemcpyHostToDevice, ctx->s) ||
-        cudaMemcpyAsync(ctx->Nsp_cal, nsp_cal.data(), g.nblk * 4, cudaMemcpyHostToDevice, ctx->s))
-        return bail(MPR_ECUDA);
     launch_build_lists(g, ctx->sl, ctx->mask, ctx->start[0], ctx->start[1], ctx->list[0],
                        ctx->list[1], ctx->split[0], ctx->split[1], ctx->s);
     ++ctx->launches;
     if (cudaMemsetAsync(ctx->sum, 0, 2 * plane * sizeof(double), ctx->s) ||
         cudaMemsetAsync(ctx->ctl, 0, sizeof(Control), ctx->s) ||
         cudaMemsetAsync(ctx->counters, 0, 4 * sizeof(unsigned long long), ctx->s) ||
-        cudaPeekAtLastError() || cudaStreamSynchronize(ctx->s))
+        cudaPeekAtLastError())
         return bail(MPR_ECUDA);
+    // (the inputs were read before the wait above; what is still queued works on
+    // the context's own memory, in its stream's order)
 #undef ST
     *out = ctx;
     return MPR_OK;
@@ -1699,11 +1634,13 @@ mpr_status mpr_get_block_stats(mpr_ctx* ctx, double* Es, int32_t* Nsp, int32_t* 
     if (!ctx) return MPR_EINVAL;
     ctx->err.clear();
     const size_t nb = ctx->g.nblk;
-    if (Es) TRY(copy_out(ctx, Es, ctx->Es, nb * 8));
-    if (Nsp) TRY(copy_out(ctx, Nsp, ctx->Nsp, nb * 4));
-    if (Nb) TRY(copy_out(ctx, Nb, ctx->Nb, nb * 4));
-    if (mean_angle) TRY(copy_out(ctx, mean_angle, ctx->init_angle, nb * 4));
-    if (n_gap) TRY(copy_out(ctx, n_gap, ctx->ngap, nb * 4));
+    // (every copy enqueued, one wait)
+    if (Es) CK(cudaMemcpyAsync(Es, ctx->Es, nb * 8, cudaMemcpyDefault, ctx->s));
+    if (Nsp) CK(cudaMemcpyAsync(Nsp, ctx->Nsp, nb * 4, cudaMemcpyDefault, ctx->s));
+    if (Nb) CK(cudaMemcpyAsync(Nb, ctx->Nb, nb * 4, cudaMemcpyDefault, ctx->s));
+    if (mean_angle) CK(cudaMemcpyAsync(mean_angle, ctx->init_angle, nb * 4, cudaMemcpyDefault, ctx->s));
+    if (n_gap) CK(cudaMemcpyAsync(n_gap, ctx->ngap, nb * 4, cudaMemcpyDefault, ctx->s));
+    CK(cudaStreamSynchronize(ctx->s));
     return MPR_OK;
 }
 

@@ -100,6 +100,19 @@ __host__ __device__ inline uint32_t local_index(const int4& rc, int y, int x) {
     return (uint32_t)(y - rc.x) * (uint32_t)rc.w + (uint32_t)(x - rc.y);
 }
 
+// Totals over a slice's blocks, and its range.
+struct SliceTotals {
+    double gsum;                          // sum of the sample angles
+    unsigned long long samples, pairs, gaps;   // samples, sample bonds, gap sites
+    double zmin, zmax;
+};
+
+// Two lists of counts and their scans (launch_scan).
+struct ScanArgs {
+    const int32_t* cnt[2];
+    int32_t* out[2];
+};
+
 struct Model {
     float q, J, inv_q;
     int overrelax;

@@ -12,6 +12,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 
 #include "mpr_device.cuh"
 #include "mpr_internal.h"
@@ -37,151 +38,237 @@ __device__ __forceinline__ uint32_t f2ord(float f) {
 
 }  // namespace
 
-float ord2f(uint32_t u) {
+__host__ __device__ float ord2f(uint32_t u) {
     uint32_t v = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
     float f;
-    __builtin_memcpy(&f, &v, 4);
+    memcpy(&f, &v, 4);
     return f;
 }
 
 // ---------------------------------------------------------------- setup --
-// z_min / z_max over the samples (Sec. 2.1: only the samples are known).
-// z_min / z_max over the samples of one field (mask != 0: gap), into mm[0..1].
-__global__ void k_minmax_field(const float* __restrict__ values, const uint8_t* __restrict__ mask,
-                               int64_t n, uint32_t* __restrict__ mm) {
-    uint32_t lo = 0xffffffffu, hi = 0u;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (mask[i]) continue;
-        const uint32_t o = f2ord(values[i]);
-        lo = min(lo, o);
-        hi = max(hi, o);
-    }
-    for (int d = 16; d > 0; d >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-    }
-    if ((threadIdx.x & 31) == 0) {
+// Inputs to canvas form and the range of the samples (Sec. 2.1: only the samples
+// are known): a field's sites get mask 1 (gap: any nonzero input) or 0, every
+// other canvas site 2 (absent); mm[2 s], mm[2 s + 1] become z_min and z_max of
+// slice s as order-preserving integers. One pass over the inputs, as the one
+// field of a context (k_prepare_field, 16 sites per thread) or by blocks
+// (k_prepare_blocks, a warp per block, which belongs to one slice).
+__device__ __forceinline__ void range_of_warp(uint32_t lo, uint32_t hi, uint32_t* mm) {
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0 && lo <= hi) {
         atomicMin(&mm[0], lo);
         atomicMax(&mm[1], hi);
     }
 }
 
-// z_min / z_max over the samples of every slice (Sec. 2.1: only the samples
-// are known): mm[2 s], mm[2 s + 1] as order-preserving integers.
-// One warp min / max per 32 sites when their samples share a slice (the
-// usual case), else an atomic per sample.
-__global__ void k_minmax(Geom g, const int32_t* __restrict__ of_block,
-                         const float* __restrict__ values, const uint8_t* __restrict__ mask,
-                         uint32_t* __restrict__ mm) {
-    const int64_t n = (int64_t)g.H * g.W;
-    const int64_t n_warps = (n + 31) / 32 * 32;   // every lane of a warp runs every iteration
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_warps;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int s = -1;
-        uint32_t lo = 0xffffffffu, hi = 0u;
-        if (i < n && !mask[i]) {
-            const int y = (int)(i / g.W), x = (int)(i % g.W);
-            s = of_block[(y / g.lb) * g.nbx + x / g.lb];
-            lo = hi = f2ord(values[i]);
-        }
-        int smax = s;
-        for (int d = 16; d > 0; d >>= 1) smax = max(smax, __shfl_xor_sync(0xffffffffu, smax, d));
-        if (__all_sync(0xffffffffu, s < 0 || s == smax)) {
-            if (smax < 0) continue;
-            for (int d = 16; d > 0; d >>= 1) {
-                lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-                hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+// kWrite: normalise the mask in place (the arrays are then 16-byte aligned);
+// otherwise only the range, of arrays aligned or not (vec: 16-byte loads allowed).
+template <bool kWrite>
+__global__ void k_prepare_field(const float* __restrict__ values, uint8_t* __restrict__ mask,
+                                int64_t n, bool vec, uint32_t* __restrict__ mm) {
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    const int64_t nv = vec ? n / 16 : 0;
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t nt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = t0; k < nv; k += nt) {
+        uint4 mw = reinterpret_cast<const uint4*>(mask)[k];
+        uint32_t w[4] = {mw.x, mw.y, mw.z, mw.w};
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const float4 v = reinterpret_cast<const float4*>(values)[4 * k + g];
+            const float f[4] = {v.x, v.y, v.z, v.w};
+            uint32_t out = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                if ((w[g] >> (8 * b)) & 0xFFu) {
+                    out |= (uint32_t)MASK_GAP << (8 * b);
+                } else {
+                    const uint32_t o = f2ord(f[b]);
+                    lo = min(lo, o);
+                    hi = max(hi, o);
+                }
             }
-            if ((threadIdx.x & 31) == 0) {
-                atomicMin(&mm[2 * smax], lo);
-                atomicMax(&mm[2 * smax + 1], hi);
-            }
-        } else if (s >= 0) {
-            atomicMin(&mm[2 * s], lo);
-            atomicMax(&mm[2 * s + 1], hi);
+            w[g] = out;
         }
+        if constexpr (kWrite)
+            reinterpret_cast<uint4*>(mask)[k] = make_uint4(w[0], w[1], w[2], w[3]);
     }
-}
-
-// Sample angles per checkerboard colour (Sec. 2.1 transform).
-__global__ void k_layout(Geom g, Slices sl, const float* __restrict__ values,
-                         const uint8_t* __restrict__ mask, float* __restrict__ dang) {
-    const int64_t n = (int64_t)g.H * g.W;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int y = (int)(i / g.W), x = (int)(i % g.W);
-        const int c = (x + y) & 1;
-        const size_t h = hidx(g, c, y, x);
+    for (int64_t i = nv * 16 + t0; i < n; i += nt) {
         if (mask[i]) {
-            dang[h] = 0.0f;
-            continue;
+            if constexpr (kWrite) mask[i] = MASK_GAP;
+        } else {
+            const uint32_t o = f2ord(values[i]);
+            lo = min(lo, o);
+            hi = max(hi, o);
         }
-        const int s = sl.of_block[(y / g.lb) * g.nbx + x / g.lb];
-        const double zmin = sl.zmin[s], zmax = sl.zmax[s];
-        const double phi = sl.degenerate[s] ? 0.0
-                                            : 6.283185307179586476925 * ((double)values[i] - zmin) /
-                                                  (zmax - zmin);
-        dang[h] = (float)phi;
+    }
+    range_of_warp(lo, hi, mm);
+}
+
+__global__ void k_prepare_blocks(Geom g, Slices sl, const float* __restrict__ values,
+                                 uint8_t* __restrict__ mask, uint32_t* __restrict__ mm) {
+    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= g.nblk) return;
+    const int y0 = (b / g.nbx) * g.lb, x0 = (b % g.nbx) * g.lb;
+    const int y1 = min(g.H, y0 + g.lb), x1 = min(g.W, x0 + g.lb);
+    const int bw = x1 - x0, nsite = (y1 - y0) * bw;
+    const int s = sl.of_block[b];
+    const int4 rc = s >= 0 ? sl.rect[s] : make_int4(0, 0, 0, 0);
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    for (int j = lane; j < nsite; j += 32) {
+        const int y = y0 + j / bw, x = x0 + j % bw;
+        const int64_t i = (int64_t)y * g.W + x;
+        uint8_t m = MASK_ABSENT;
+        if (y < rc.x + rc.z && x < rc.y + rc.w) {
+            m = mask[i] != 0 ? MASK_GAP : 0;
+            if (m == 0) {
+                const uint32_t o = f2ord(values[i]);
+                lo = min(lo, o);
+                hi = max(hi, o);
+            }
+        }
+        mask[i] = m;
+    }
+    if (s >= 0) range_of_warp(lo, hi, mm + 2 * s);
+}
+
+// Slice ranges as numbers, and cleared totals: one thread per slice.
+__global__ void k_slice_range(int n, const uint32_t* __restrict__ mm, double* __restrict__ zmin,
+                              double* __restrict__ zmax, int32_t* __restrict__ degenerate,
+                              SliceTotals* __restrict__ tot) {
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
+        const bool any = mm[2 * s] != 0xffffffffu;   // the slice has a sample
+        const double lo = any ? (double)ord2f(mm[2 * s]) : 0.0;
+        const double hi = any ? (double)ord2f(mm[2 * s + 1]) : 0.0;
+        zmin[s] = lo;
+        zmax[s] = hi;
+        degenerate[s] = !(hi > lo);
+        tot[s] = SliceTotals{0.0, 0, 0, 0, lo, hi};
     }
 }
 
-// One warp per block: Eq. 2 over the owned sample-sample bonds (FP64), bond
-// counts, sample mean angle, gap counts per colour.
-__global__ void k_block_stats(Geom g, Slices sl, const float* __restrict__ values,
-                              const uint8_t* __restrict__ mask, double q, double J,
-                              double* __restrict__ Es, int32_t* __restrict__ Nsp,
-                              int32_t* __restrict__ Nb, double* __restrict__ ssum,
-                              int32_t* __restrict__ nsamp, int32_t* __restrict__ ngap0,
-                              int32_t* __restrict__ ngap1) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= g.nblk) return;
-    const int by = warp / g.nbx, bx = warp % g.nbx;
+// One CTA per block: Eq. 2 over the owned sample-sample bonds (FP64), bond
+// counts, sample mean angle, gap counts per colour, the sites' sample angles
+// (Sec. 2.1 transform), and the slice's totals.
+__global__ void __launch_bounds__(32 * kStatsMaxWarps)
+k_block_stats(Geom g, Slices sl, const float* __restrict__ values,
+              const uint8_t* __restrict__ mask, double q, double J, double* __restrict__ Es,
+              int32_t* __restrict__ Nsp, int32_t* __restrict__ Nb, double* __restrict__ ssum,
+              int32_t* __restrict__ nsamp, int32_t* __restrict__ ngap0,
+              int32_t* __restrict__ ngap1, float* __restrict__ dang,
+              SliceTotals* __restrict__ tot) {
+    __shared__ StatsShared sh;
+    const int b = blockIdx.x;
+    const int by = b / g.nbx, bx = b % g.nbx;
     const int y0 = by * g.lb, x0 = bx * g.lb;
     const int y1 = min(g.H, y0 + g.lb), x1 = min(g.W, x0 + g.lb);
-    const int s = sl.of_block[warp];
+    const int s = sl.of_block[b];
     const double zmin = s >= 0 ? sl.zmin[s] : 0.0, zmax = s >= 0 ? sl.zmax[s] : 1.0;
     const double scale = (s < 0 || sl.degenerate[s]) ? 0.0 : 6.283185307179586476925 / (zmax - zmin);
     // A bond to the right / down neighbour exists when that site is present
     // and in the same slice (blocks never straddle slices).
-    const bool right_ok = x1 < g.W && bx + 1 < g.nbx && sl.of_block[warp + 1] == s;
-    const bool down_ok = y1 < g.H && by + 1 < g.nby && sl.of_block[warp + g.nbx] == s;
+    const bool right_ok = x1 < g.W && bx + 1 < g.nbx && sl.of_block[b + 1] == s;
+    const bool down_ok = y1 < g.H && by + 1 < g.nby && sl.of_block[b + g.nbx] == s;
     const BlockSums r = block_sums<true>(values, mask, g.W, y0, x0, y1, x1, right_ok, down_ok,
-                                         zmin, scale, q, J, s >= 0);
-    if (lane == 0) {
-        Es[warp] = r.es;
-        Nsp[warp] = r.nsp;
-        Nb[warp] = r.nb;
-        ssum[warp] = r.sm;
-        nsamp[warp] = r.ns;
-        ngap0[warp] = r.g0;
-        ngap1[warp] = r.g1;
+                                         zmin, zmax, scale, q, J, s >= 0, dang, g.Wh,
+                                         (size_t)g.H * g.Wh, sh);
+    if (threadIdx.x != 0) return;
+    Es[b] = r.es;
+    Nsp[b] = r.nsp;
+    Nb[b] = r.nb;
+    ssum[b] = r.sm;
+    nsamp[b] = r.ns;
+    ngap0[b] = r.g0;
+    ngap1[b] = r.g1;
+    if (s < 0) return;
+    if (r.ns) {
+        atomicAdd(&tot[s].gsum, r.sm);
+        atomicAdd(&tot[s].samples, (unsigned long long)r.ns);
+    }
+    if (r.nsp) atomicAdd(&tot[s].pairs, (unsigned long long)r.nsp);
+    if (r.g0 + r.g1) atomicAdd(&tot[s].gaps, (unsigned long long)(r.g0 + r.g1));
+}
+
+// What the samples alone decide about every block: e_s,b (0 without sample
+// bonds), 1 / N_b, gap sites, sample bonds of the blocks that calibrate (those
+// with gap sites), and the start angle (Sec. 3.3.3): the block's mean sample
+// angle, the slice's where the block has no sample.
+__global__ void k_block_finish(int nblk, const int32_t* __restrict__ of_block,
+                               const double* __restrict__ Es, const int32_t* __restrict__ Nsp,
+                               const int32_t* __restrict__ Nb, const double* __restrict__ ssum,
+                               const int32_t* __restrict__ nsamp,
+                               const int32_t* __restrict__ ngap0,
+                               const int32_t* __restrict__ ngap1,
+                               const SliceTotals* __restrict__ tot, double* __restrict__ es,
+                               double* __restrict__ inb, int32_t* __restrict__ ngap,
+                               int32_t* __restrict__ Nsp_cal, float* __restrict__ init) {
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nblk; b += gridDim.x * blockDim.x) {
+        const int n = ngap0[b] + ngap1[b], nsp = Nsp[b], s = of_block[b];
+        es[b] = nsp > 0 ? Es[b] / (double)nsp : 0.0;
+        inb[b] = Nb[b] > 0 ? 1.0 / (double)Nb[b] : 0.0;
+        ngap[b] = n;
+        Nsp_cal[b] = n > 0 ? nsp : 0;
+        float a = 0.0f;
+        if (nsamp[b] > 0) a = (float)(ssum[b] / (double)nsamp[b]);
+        else if (s >= 0 && tot[s].samples > 0) a = (float)(tot[s].gsum / (double)tot[s].samples);
+        init[b] = s >= 0 ? a : 0.0f;
     }
 }
 
-// Exclusive scan of n counts into out[0..n] by one CTA of 1024 threads.
-__global__ void k_scan_counts(const int32_t* __restrict__ cnt, int n, int32_t* __restrict__ out) {
-    __shared__ int64_t part[1024];
-    const int t = threadIdx.x;
-    const int per = (n + 1023) / 1024;
-    const int a = min(n, t * per), b = min(n, a + per);
+// Exclusive scans of n counts into out[0..n], one CTA of 1024 threads per list
+// (blockIdx.x). A thread reads its run of counts four at a time: the reads of
+// one after the other, 16 per thread at 16 k blocks, took 17 us.
+__global__ void k_scan_counts(ScanArgs a, int n) {
+    __shared__ int64_t part[32];
+    const int32_t* __restrict__ cnt = a.cnt[blockIdx.x];
+    int32_t* __restrict__ out = a.out[blockIdx.x];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = ((n + 1023) / 1024 + 3) / 4 * 4;
+    const int64_t first = (int64_t)t * per;
+    const int i0 = (int)(first < n ? first : n), i1 = (int)(first + per < n ? first + per : n);
+    auto each = [&](auto&& f) {
+        for (int i = i0; i < i1; i += 4) {
+            int4 v = make_int4(0, 0, 0, 0);
+            if (i + 4 <= i1) {
+                v = *reinterpret_cast<const int4*>(cnt + i);
+            } else {
+                v.x = cnt[i];
+                if (i + 1 < i1) v.y = cnt[i + 1];
+                if (i + 2 < i1) v.z = cnt[i + 2];
+            }
+            f(i, v);
+        }
+    };
     int64_t s = 0;
-    for (int i = a; i < b; ++i) s += cnt[i];
-    part[t] = s;
+    each([&](int, const int4& v) { s += (int64_t)v.x + v.y + v.z + v.w; });
+    int64_t run = s;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, run, d);
+        if (lane >= d) run += u;
+    }
+    if (lane == 31) part[warp] = run;
     __syncthreads();
-    for (int d = 1; d < 1024; d <<= 1) {
-        int64_t v = t >= d ? part[t - d] : 0;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
+    if (warp == 0) {
+        int64_t p = part[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int64_t u = __shfl_up_sync(0xffffffffu, p, d);
+            if (lane >= d) p += u;
+        }
+        part[lane] = p;
     }
-    int64_t run = part[t] - s;
-    for (int i = a; i < b; ++i) {
-        out[i] = (int32_t)run;
-        run += cnt[i];
-    }
-    if (t == 1023) out[n] = (int32_t)part[1023];
+    __syncthreads();
+    run += (warp ? part[warp - 1] : 0) - s;   // the counts before this thread's
+    each([&](int i, const int4& v) {
+        const int32_t c[4] = {v.x, v.y, v.z, v.w};
+        for (int k = 0; k < 4 && i + k < i1; ++k) {
+            out[i + k] = (int32_t)run;
+            run += c[k];
+        }
+    });
+    if (t == 1023) out[n] = (int32_t)part[31];
 }
 
 // One warp per block: write the gap entries of both colours into the block's
@@ -1054,32 +1141,61 @@ inline int grid_for(int64_t n, int threads, int max_blocks = 152 * 16) {
 }
 }  // namespace
 
+namespace {
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+}  // namespace
+
 void launch_minmax_field(const float* values, const uint8_t* mask, int64_t n, uint32_t* mm,
                          cudaStream_t s) {
-    k_minmax_field<<<grid_for(n, 256), 256, 0, s>>>(values, mask, n, mm);
+    const bool vec = aligned16(values) && aligned16(mask);
+    k_prepare_field<false><<<grid_for(vec ? n / 16 + 1 : n, 256), 256, 0, s>>>(
+        values, const_cast<uint8_t*>(mask), n, vec, mm);
 }
 
-void launch_minmax(const Geom& g, const int32_t* of_block, const float* values,
-                   const uint8_t* mask, uint32_t* mm, cudaStream_t s) {
-    k_minmax<<<grid_for((int64_t)g.H * g.W, 256), 256, 0, s>>>(g, of_block, values, mask, mm);
+void launch_prepare(const Geom& g, const Slices& sl, const float* values, uint8_t* mask,
+                    uint32_t* mm, cudaStream_t s) {
+    const int64_t n = (int64_t)g.H * g.W;
+    if (sl.n == 1 && sl.rect0.x == 0 && sl.rect0.y == 0 && sl.rect0.z == g.H && sl.rect0.w == g.W) {
+        const bool vec = aligned16(values) && aligned16(mask);
+        k_prepare_field<true><<<grid_for(vec ? n / 16 + 1 : n, 256), 256, 0, s>>>(values, mask, n,
+                                                                                 vec, mm);
+    } else {
+        k_prepare_blocks<<<(unsigned)(((int64_t)g.nblk * 32 + 255) / 256), 256, 0, s>>>(
+            g, sl, values, mask, mm);
+    }
 }
 
-void launch_layout(const Geom& g, const Slices& sl, const float* values, const uint8_t* mask,
-                   float* dang, cudaStream_t s) {
-    k_layout<<<grid_for((int64_t)g.H * g.W, 256), 256, 0, s>>>(g, sl, values, mask, dang);
+void launch_slice_range(int n, const uint32_t* mm, double* zmin, double* zmax,
+                        int32_t* degenerate, SliceTotals* tot, cudaStream_t s) {
+    k_slice_range<<<grid_for(n, 256), 256, 0, s>>>(n, mm, zmin, zmax, degenerate, tot);
 }
+
+// Threads per block of the grid: enough CTAs in flight on large grids with 128,
+// shorter per-thread chains on grids of few blocks with 256 (both sides measured
+// at 256^2, l_b = 16 and 4096^2, l_b = 32).
+int stats_threads(int nblk) { return nblk < 152 * 8 ? 256 : 128; }
 
 void launch_block_stats(const Geom& g, const Slices& sl, const float* values, const uint8_t* mask,
                         double q, double J, double* Es, int32_t* Nsp, int32_t* Nb, double* ssum,
-                        int32_t* nsamp, int32_t* ngap0, int32_t* ngap1, cudaStream_t s) {
-    const int threads = 256;
-    const int blocks = (int)(((int64_t)g.nblk * 32 + threads - 1) / threads);
-    k_block_stats<<<blocks, threads, 0, s>>>(g, sl, values, mask, q, J, Es, Nsp, Nb, ssum, nsamp,
-                                             ngap0, ngap1);
+                        int32_t* nsamp, int32_t* ngap0, int32_t* ngap1, float* dang,
+                        SliceTotals* tot, cudaStream_t s) {
+    k_block_stats<<<g.nblk, stats_threads(g.nblk), 0, s>>>(g, sl, values, mask, q, J, Es, Nsp, Nb,
+                                                           ssum, nsamp, ngap0, ngap1, dang, tot);
 }
 
-void launch_scan(const int32_t* cnt, int n, int32_t* out, cudaStream_t s) {
-    k_scan_counts<<<1, 1024, 0, s>>>(cnt, n, out);
+void launch_block_finish(int nblk, const int32_t* of_block, const double* Es, const int32_t* Nsp,
+                         const int32_t* Nb, const double* ssum, const int32_t* nsamp,
+                         const int32_t* ngap0, const int32_t* ngap1, const SliceTotals* tot,
+                         double* es, double* inb, int32_t* ngap, int32_t* Nsp_cal, float* init,
+                         cudaStream_t s) {
+    k_block_finish<<<grid_for(nblk, 256), 256, 0, s>>>(nblk, of_block, Es, Nsp, Nb, ssum, nsamp,
+                                                      ngap0, ngap1, tot, es, inb, ngap, Nsp_cal,
+                                                      init);
+}
+
+void launch_scan(const int32_t* cnt0, const int32_t* cnt1, int n, int32_t* out0, int32_t* out1,
+                 cudaStream_t s) {
+    k_scan_counts<<<2, 1024, 0, s>>>(ScanArgs{{cnt0, cnt1}, {out0, out1}}, n);
 }
 
 void launch_build_lists(const Geom& g, const Slices& sl, const uint8_t* mask,

@@ -8,20 +8,29 @@
 
 namespace mpr {
 
-float ord2f(uint32_t u);
+__host__ __device__ float ord2f(uint32_t u);
 
 // One field (mask != 0: gap): mm[0..1] = order-preserving (min, max), pre-set.
 void launch_minmax_field(const float* values, const uint8_t* mask, int64_t n, uint32_t* mm,
                          cudaStream_t s);
 // mm: 2 per slice (order-preserving min, max), pre-set to (max, 0).
-void launch_minmax(const Geom& g, const int32_t* of_block, const float* values,
-                   const uint8_t* mask, uint32_t* mm, cudaStream_t s);
-void launch_layout(const Geom& g, const Slices& sl, const float* values, const uint8_t* mask,
-                   float* dang, cudaStream_t s);
+void launch_prepare(const Geom& g, const Slices& sl, const float* values, uint8_t* mask,
+                    uint32_t* mm, cudaStream_t s);
+void launch_slice_range(int n, const uint32_t* mm, double* zmin, double* zmax,
+                        int32_t* degenerate, SliceTotals* tot, cudaStream_t s);
+int stats_threads(int nblk);
 void launch_block_stats(const Geom& g, const Slices& sl, const float* values, const uint8_t* mask,
                         double q, double J, double* Es, int32_t* Nsp, int32_t* Nb, double* ssum,
-                        int32_t* nsamp, int32_t* ngap0, int32_t* ngap1, cudaStream_t s);
-void launch_scan(const int32_t* cnt, int n, int32_t* out, cudaStream_t s);
+                        int32_t* nsamp, int32_t* ngap0, int32_t* ngap1, float* dang,
+                        SliceTotals* tot, cudaStream_t s);
+void launch_block_finish(int nblk, const int32_t* of_block, const double* Es, const int32_t* Nsp,
+                         const int32_t* Nb, const double* ssum, const int32_t* nsamp,
+                         const int32_t* ngap0, const int32_t* ngap1, const SliceTotals* tot,
+                         double* es, double* inb, int32_t* ngap, int32_t* Nsp_cal, float* init,
+                         cudaStream_t s);
+// The counts of two lists (16-byte aligned), each scanned into out[0..n].
+void launch_scan(const int32_t* cnt0, const int32_t* cnt1, int n, int32_t* out0, int32_t* out1,
+                 cudaStream_t s);
 void launch_build_lists(const Geom& g, const Slices& sl, const uint8_t* mask,
                         const int32_t* start0, const int32_t* start1, uint4* list0, uint4* list1,
                         int32_t* split0, int32_t* split1, cudaStream_t s);
