@@ -2160,13 +2160,14 @@ mpr_status simulate_tail(mpr_ctx* ctx, bool* ran) {
     return MPR_OK;
 }
 
-// The rest of the sweep loop with one CTA per realization pair (the stop
+// The rest of the sweep loop with one cluster per realization pair (the stop
 // tail, once every pair's running units fit one CTA's buffer).
 mpr_status simulate_pair_tail(mpr_ctx* ctx) {
     const SimTailArgs a = tail_args(ctx);
     TailProfile tp;
     TRY(tail_profile_begin(ctx, tp));
-    const cudaError_t le = launch_pair_tail(a, ctx->storage, ctx->Rp / 2, ctx->s);
+    const int ctas = pair_tail_ctas(ctx->storage, ctx->Rp / 2);
+    const cudaError_t le = launch_pair_tail(a, ctx->storage, ctx->Rp / 2, ctas, ctx->s);
     if (le != cudaSuccess) return fail(ctx, MPR_ECUDA, "stop tail: %s", cudaGetErrorString(le));
     ++ctx->launches;
     TRY(tail_profile_end(ctx, tp));

@@ -151,7 +151,9 @@ cudaError_t launch_sim_tail(const SimTailArgs& a, int storage, int grid, cudaStr
 // The realizations' stop tail with one CTA per realization pair
 // (mpr_pairtail.cu); every pair's running units must fit kPairTailCap.
 constexpr int kPairTailCap = 4096;
-cudaError_t launch_pair_tail(const SimTailArgs& a, int storage, int n_pairs,
+// CTAs per cluster: the most that keep every pair's cluster resident.
+int pair_tail_ctas(int storage, int n_pairs);
+cudaError_t launch_pair_tail(const SimTailArgs& a, int storage, int n_pairs, int ctas,
                              cudaStream_t s);
 
 // The staged half-step (mpr_tile.cu): tile shape of a geometry, the staging
