@@ -1286,9 +1286,8 @@ void launch_sweep_flat(const SweepArgs& a, int G, int64_t n_list, cudaStream_t s
     FoldArgs f{};
     if (fold) f = *fold;
     if (n_list == 0 && f.ctas == 0) return;
-    const int64_t threads = n_list * (G / 2);
-    const dim3 grid((unsigned)((threads + kFlatThreads - 1) / kFlatThreads + f.ctas),
-                    (unsigned)a.groups);
+    const dim3 grid((unsigned)((n_list + kFlatThreads - 1) / kFlatThreads + f.ctas),
+                    (unsigned)((a.R + 1) / 2));
     // Programmatic dependent launch: this half-step's prologue overlaps the
     // previous launch's tail (the kernel waits before touching its output).
     if (G == 2) launch_pdl(k_sweep_flat<2>, grid, kFlatThreads, s, a, n_list, f);

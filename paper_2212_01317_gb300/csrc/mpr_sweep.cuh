@@ -490,9 +490,8 @@ __device__ __forceinline__ void sweep_item_half(const SweepArgs& a, int b, int p
 }
 
 // One half-step over the whole list of one colour, flat: one thread per
-// (gap entry, realization pair), 32 / (G/2) entries per warp, one lane group
-// per blockIdx.y (a CTA never mixes lane groups). For calibration, where every
-// block runs and only one or a few chains exist, this puts every site's
+// (gap entry, realization pair). For calibration, where every block runs
+// and only one or a few chains exist, this puts every site's
 // latency chain into one wave. The block-energy change is summed per CTA in
 // shared memory (the list is block-major, so a CTA spans few blocks) and
 // flushed with one atomic per (block, realization); changes that belong to
@@ -515,19 +514,28 @@ __device__ __forceinline__ void grid_dep_launch() {
 // The list entry, its Philox block and the temperatures do not depend on the
 // previous half-step, so they are taken before the dependency wait and
 // overlap the previous launch's tail.
+//
+// A CTA takes kFlatThreads entries of one pair (blockIdx.y), so no thread is
+// left to the padding lanes of a group of G; the sums keep the group's shares:
+// G / 2 sections of a CTA, each with shared-memory sums of its own, and warp
+// sums of 64 / G entries. With an entry's G / 2 pairs on neighbouring threads,
+// four chains (G = 8) left half of the threads idle: forward and backward of a
+// 1024^2 field 2.85 ms, now 2.17; three chains 3.15 -> 2.05, eight (no padding)
+// 3.07 -> 3.10.
 template <int G>
 __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, uint32_t ctr1) {
-    constexpr int NP = G / 2;
-    __shared__ float acc[kFlatBlocks * G];
-    const int grp = blockIdx.y;
-    const int64_t t0 = (int64_t)blockIdx.x * kFlatThreads;
-    const int64_t t = t0 + threadIdx.x;
-    const int64_t e = t / NP;
-    const int q = (int)(t % NP);
-    for (int i = threadIdx.x; i < kFlatBlocks * G; i += kFlatThreads) acc[i] = 0.0f;
-    const int b0 = (int)(a.list[t0 / NP].y >> META_SHIFT);
+    constexpr int kSections = G / 2;
+    constexpr int kSection = kFlatThreads / kSections;
+    constexpr int kSum = 32 / kSections;
+    __shared__ float acc[kSections][kFlatBlocks * 2];
+    const int sec = (int)threadIdx.x / kSection;
+    const int64_t e0 = (int64_t)blockIdx.x * kFlatThreads;
+    const int64_t e = e0 + threadIdx.x;
+    for (int i = threadIdx.x; i < kSections * kFlatBlocks * 2; i += kFlatThreads) (&acc[0][0])[i] = 0.0f;
+    const int64_t s0 = e0 + sec * kSection;
+    const int b0 = kSections == 1 || s0 < n_list ? (int)(a.list[s0].y >> META_SHIFT) : 0;
     const bool live = e < n_list;
-    const int rl = grp * G + 2 * q;
+    const int rl = 2 * (int)blockIdx.y;
     uint4 en = make_uint4(0u, 0u, 0u, 0u);
     int b = b0;
     uint32_t w[4] = {0u, 0u, 0u, 0u};
@@ -575,36 +583,36 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
         }
     }
     if (!a.energy) return;
-    // The block's share: one warp sum per realization lane when the warp's
-    // entries all lie in one block (the usual case: the list is block-major),
-    // else an atomic per lane; shared-memory sums for the CTA's first blocks.
+    // The block's share: one sum per realization when all kSum entries lie in
+    // one block (the usual case: the list is block-major), else an atomic per
+    // lane; shared-memory sums for the section's first blocks.
     const int lane = threadIdx.x & 31;
-    if (__all_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, 0))) {
+    const int first = lane & ~(kSum - 1);
+    bool whole;
+    float2 sum = ao;
+    if constexpr (kSections == 1) {
+        whole = __all_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, 0));
+    } else {
+        const uint32_t same = __ballot_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, first));
+        whole = ((same >> first) & ((1u << (kSum & 31)) - 1u)) == (1u << (kSum & 31)) - 1u;
+    }
+    if (kSections > 1 || whole) {
 #pragma unroll
-        for (int d = 16; d >= NP; d >>= 1) {
-            ao.x += __shfl_xor_sync(0xffffffffu, ao.x, d);
-            ao.y += __shfl_xor_sync(0xffffffffu, ao.y, d);
+        for (int d = kSum / 2; d >= 1; d >>= 1) {
+            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, d);
+            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, d);
         }
-        if (lane < NP) {
-            const int loc = b - b0;
-            if (loc < kFlatBlocks) {
-                if (ao.x != 0.0f) atomicAdd(&acc[loc * G + 2 * lane], ao.x);
-                if (ao.y != 0.0f) atomicAdd(&acc[loc * G + 2 * lane + 1], ao.y);
-            } else {
-                double* ea = a.eacc + (size_t)b * a.Rp + grp * G + 2 * lane;
-                if (ao.x != 0.0f) atomicAdd(ea, (double)ao.x);
-                if (ao.y != 0.0f) atomicAdd(ea + 1, (double)ao.y);
-            }
-        }
-    } else if (live) {
+    }
+    if (whole ? lane == first : live) {
+        if (!whole) sum = ao;
         const int loc = b - b0;
         if (loc < kFlatBlocks) {
-            if (ao.x != 0.0f) atomicAdd(&acc[loc * G + 2 * q], ao.x);
-            if (ao.y != 0.0f) atomicAdd(&acc[loc * G + 2 * q + 1], ao.y);
+            if (sum.x != 0.0f) atomicAdd(&acc[sec][loc * 2], sum.x);
+            if (sum.y != 0.0f) atomicAdd(&acc[sec][loc * 2 + 1], sum.y);
         } else {
             double* ea = a.eacc + (size_t)b * a.Rp + rl;
-            if (ao.x != 0.0f) atomicAdd(ea, (double)ao.x);
-            if (ao.y != 0.0f) atomicAdd(ea + 1, (double)ao.y);
+            if (sum.x != 0.0f) atomicAdd(ea, (double)sum.x);
+            if (sum.y != 0.0f) atomicAdd(ea + 1, (double)sum.y);
         }
     }
     // Left / up bonds of edge sites belong to the neighbouring blocks.
@@ -617,9 +625,9 @@ __device__ __forceinline__ void sweep_flat(const SweepArgs& a, int64_t n_list, u
         if (au.y != 0.0f) atomicAdd(ea - up + 1, (double)au.y);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kFlatBlocks * G; i += kFlatThreads) {
-        const float v = acc[i];
-        if (v != 0.0f) atomicAdd(&a.eacc[(size_t)(b0 + i / G) * a.Rp + grp * G + (i % G)], (double)v);
+    for (int i = (int)threadIdx.x % kSection; i < kFlatBlocks * 2; i += kSection) {
+        const float v = acc[sec][i];
+        if (v != 0.0f) atomicAdd(&a.eacc[(size_t)(b0 + i / 2) * a.Rp + rl + (i & 1)], (double)v);
     }
 }
 
