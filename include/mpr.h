@@ -85,14 +85,16 @@ typedef struct {
                             to the stored type before their energy is taken, so the
                             incremental block energies stay exact for the stored state.
                             Sample angles and the calibration chains stay FP32. */
-    int32_t group;       /* realizations interleaved per site: 0 = auto, 2 or 8 */
+    int32_t group;       /* realizations per lane group (padding and block sums): 0 = auto,
+                            2 or 8 */
     int32_t profile;     /* 1: time every sweep-kernel launch with CUDA events (default 0) */
-    int32_t cal_mode;    /* calibration launch: 0 auto (= 1), 1 one CUDA graph of per-half-step
+    int32_t cal_mode;    /* calibration launch: 0 auto (= 1), 1 one CUDA graph of an iteration's
                             launches, 2 one persistent cooperative kernel with grid barriers,
                             3 every kernel launched from the host (profilers see each one;
-                            with profile = 1 every half-step is timed) */
-    int32_t wait_ms;     /* limit of a device-side grid-barrier wait (default 2000 ms);
-                            a wait that gives up makes the call return MPR_ETIMEOUT */
+                            with profile = 1 every half-step launch is timed) */
+    int32_t wait_ms;     /* limit of a device-side wait between CTAs (default 2000 ms); a wait
+                            that gives up makes the call return MPR_ETIMEOUT, or mpr_calibrate
+                            run again with a launch per half-step where it chose another form */
     int32_t barrier_test; /* test hook: extra arrivals the grid barrier waits for (default 0);
                              > 0 makes every wait give up after wait_ms */
     int32_t cal_method;  /* 0 bisection (default), 1 damped Newton steps on beta_b with
@@ -162,12 +164,15 @@ typedef struct {
                              n_meas measured ones. Needs cal_method 0 and a cal_mode other
                              than 2 */
     int32_t cal_sweep;   /* form of the calibration's half-steps (cal_mode 1 and 3): 0 (default)
-                            picks by size: one warp per (block, realization pair) when a
+                            picks by size: an iteration's half-steps in one launch while the
+                            gap sites fit a cluster's or the GPU's shared memory (chains that
+                            restart every iteration); else one warp per (block, realization
+                            pair) when a
                             colour's list needs 2^20 or more threads in the other form and the
                             grid holds at least 64 such units per SM, else one thread per (gap
                             entry, realization pair); 1 always the latter, 2 always the former.
-                            Both compute the same moves from the same random numbers; only the
-                            FP32 order of the block sums differs */
+                            All compute the same moves from the same random numbers; only the
+                            order of the block sums differs */
     void* cuda_stream;   /* cudaStream_t to issue work on (NULL = default stream) */
 } mpr_options;
 

@@ -140,6 +140,16 @@ struct mpr_ctx {
     float* med = nullptr;
     int coop = 0;                // device supports cooperative launch
     int cal_clusters = -1;       // cal_cluster_max_active() (-1: not asked yet)
+    // The resident calibration (mpr_calresident.cu): whether the running
+    // mpr_calibrate uses it, whether it has been given up on, its plan for
+    // res_ctas CTAs per pair, and its workspaces.
+    bool resident = false, res_refused = false;
+    int res_ctas = 0;
+    CalResidentPlan res_plan{};
+    int* res_part = nullptr;          // [2][kCalResidentCtas + 1] and the plan
+    float4* res_sync = nullptr;       // the error and arrival words, then the exports
+    size_t res_cap = 0;
+    CalResidentArgs res{};
 
     int64_t realizations = 0;   // accumulated into sum
     int64_t r_next = 0;         // index of the next realization
@@ -871,7 +881,8 @@ bool cluster_calibration(mpr_ctx* ctx) {
     return ctx->Rp / 2 <= kCalClusterRounds * ctx->cal_clusters;
 }
 
-mpr_status cluster_sweeps(mpr_ctx* ctx, bool timed) {
+// The arguments both one-launch forms of an iteration share.
+CalClusterArgs cal_args(mpr_ctx* ctx) {
     const mpr_options& o = ctx->opt;
     CalClusterArgs a{};
     a.sw = sweep_args(ctx, 0, false);
@@ -892,13 +903,97 @@ mpr_status cluster_sweeps(mpr_ctx* ctx, bool timed) {
     a.ebar = ctx->ebar;
     a.ebar_odd = ctx->ebar2;
     a.ebar_pts = ctx->ebark;
+    return a;
+}
+
+// Decides (outside any capture) whether this calibration's iterations run as
+// one cooperative launch each (mpr_calresident.cu), and prepares it: restarting
+// chains, the automatic half-step form, more gap sites than the cluster form
+// takes, and at most kCalResidentSites per colour and CTA, with what their
+// updates read, in the shared memory of the CTAs a pair gets. It was faster at
+// every size it takes (24 bisections, one chain, half of the sites missing:
+// 256^2 7.6 -> 4.8 ms, 512^2 11.4 -> 5.2, 1024^2 12.9 -> 9.8; 700^2, four points,
+// 8 iterations 8.7 -> 4.5). Beyond it a half-step per launch streams the lists
+// in several waves and the launch weighs little. A CTA gets at least
+// kCalResidentMin sites of a colour (with 512, 256^2 took 3 % longer).
+constexpr int kCalResidentMin = 256;
+
+mpr_status prepare_resident(mpr_ctx* ctx) {
+    const mpr_options& o = ctx->opt;
+    ctx->resident = false;
+    const int64_t most = std::max(ctx->n_gap[0], ctx->n_gap[1]);
+    const int pairs = (ctx->R + 1) / 2;
+    const bool cluster = cluster_calibration(ctx);
+    if (cluster || ctx->res_refused || o.cal_sweep != 0 || o.cal_continue >= 0 || o.cal_mode == 2 ||
+        o.n_bisect <= 0 || !ctx->coop || ctx->n_gap[0] == 0 || ctx->n_gap[1] == 0)
+        return MPR_OK;
+    const int ctas = (int)std::min<int64_t>(std::min(ctx->n_sm / pairs, kCalResidentCtas),
+                                            (most + kCalResidentMin - 1) / kCalResidentMin);
+    if (ctas < 1 || most > (int64_t)ctas * kCalResidentSites) return MPR_OK;
+    const size_t smem = cal_resident_smem_max(ctx->device);
+    if (smem == 0) return MPR_OK;
+    constexpr size_t kPart = 2 * (kCalResidentCtas + 1);
+    if (ctx->res_ctas != ctas) {
+        if (!ctx->res_part) TRY(dalloc(ctx, &ctx->res_part, kPart + sizeof(CalResidentPlan) / 4));
+        ctx->res_ctas = 0;
+        launch_cal_resident_plan(ctx->list, ctx->start, ctx->n_gap, ctas, ctx->res_part,
+                                 ctx->res_part + kPart, ctx->s);
+        CKL();
+        CK(cudaMemcpyAsync(&ctx->res_plan, ctx->res_part + kPart, sizeof(CalResidentPlan),
+                           cudaMemcpyDeviceToHost, ctx->s));
+        CK(cudaStreamSynchronize(ctx->s));
+        ctx->res_ctas = ctas;
+    }
+    const CalResidentPlan& plan = ctx->res_plan;
+    CalResidentArgs a{};
+    a.part = ctx->res_part;
+    a.ctas = ctas;
+    a.cap = (plan.most + 31) / 32 * 32;
+    a.sites = plan.sites;
+    a.consts = (plan.consts + 2) / 2 * 2;       // (one more: no neighbour)
+    a.edges = plan.edges;
+    a.blocks = plan.blocks;
+    if (a.cap > kCalResidentSites || a.edges > 2048 || a.blocks > 2048) return MPR_OK;
+    const size_t fixed = cal_resident_smem(a);
+    if (fixed >= smem) return MPR_OK;
+    a.halo = 2;
+    const size_t per_two = cal_resident_smem(a) - fixed;
+    a.halo = (int)std::min<size_t>(1024, (smem - fixed) / per_two * 2);
+    if (a.halo < 32 || 2 * (a.sites + 2 * a.halo) + a.consts > 0x10000) return MPR_OK;
+    const size_t need = 1 + (size_t)pairs * ctas * 2 * a.cap;
+    if (need > ctx->res_cap) {
+        dfree(ctx, ctx->res_sync);
+        ctx->res_sync = nullptr;
+        ctx->res_cap = 0;
+        TRY(dalloc(ctx, &ctx->res_sync, need));
+        ctx->res_cap = need;
+    }
+    CK(cudaMemsetAsync(ctx->res_sync, 0, sizeof(uint32_t), ctx->s));
+    a.sync = reinterpret_cast<uint32_t*>(ctx->res_sync);
+    a.exports = ctx->res_sync + 1;
+    a.arrivals = (uint32_t)(pairs * ctas + o.barrier_test);
+    a.spin_limit = (uint32_t)std::min<int64_t>((int64_t)o.wait_ms * 1000, 0xffffffff);  // ~1 us a poll
+    ctx->res = a;
+    ctx->resident = true;
+    return MPR_OK;
+}
+
+// An iteration's sweeps in one launch, of the cluster or the resident form.
+mpr_status one_launch_sweeps(mpr_ctx* ctx, bool timed) {
+    const CalClusterArgs a = cal_args(ctx);
+    if (ctx->resident) {
+        ctx->res.cal = a;
+        const size_t words = (size_t)((ctx->R + 1) / 2) * ctx->res.ctas * 2 * ctx->res.cap;
+        CK(cudaMemsetAsync(ctx->res.sync + 1, 0, sizeof(float4) * (1 + words) - sizeof(uint32_t),
+                           ctx->s));
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (timed && o.profile) {
+    if (timed && ctx->opt.profile) {
         e0 = get_event(ctx);
         e1 = get_event(ctx);
         if (e0) cudaEventRecord(e0, ctx->s);
     }
-    CK(launch_cal_cluster(a, ctx->s));
+    CK(ctx->resident ? launch_cal_resident(ctx->res, ctx->s) : launch_cal_cluster(a, ctx->s));
     if (e0 && e1) {
         cudaEventRecord(e1, ctx->s);
         ctx->ev_cal.emplace_back(e0, e1);
@@ -951,8 +1046,8 @@ mpr_status calibration_iteration(mpr_ctx* ctx, double inv_count, cudaGraphCondit
     }
     const size_t blk = (size_t)g.nblk * ctx->Rp;
     const bool restart = first || o.cal_continue < 0;
-    if (cluster_calibration(ctx)) {
-        TRY(cluster_sweeps(ctx, timed));
+    if (ctx->resident || cluster_calibration(ctx)) {
+        TRY(one_launch_sweeps(ctx, timed));
         return cal_update(ctx, inv_count, cond);
     }
     if (restart) {
@@ -1712,10 +1807,9 @@ mpr_status mpr_set_energy_curve(mpr_ctx* ctx, const float* T, const double* e, i
     return MPR_OK;
 }
 
-mpr_status mpr_calibrate(mpr_ctx* ctx, float* block_T_out) {
-    PhaseRange phase_range("mpr_calibrate");
-    if (!ctx) return MPR_EINVAL;
+static mpr_status calibrate(mpr_ctx* ctx, float* block_T_out) {
     ctx->err.clear();
+    ctx->resident = false;
     const Geom& g = ctx->g;
     const mpr_options& o = ctx->opt;
     ctx->batch_open = 0;
@@ -1782,7 +1876,7 @@ mpr_status mpr_calibrate(mpr_ctx* ctx, float* block_T_out) {
     launch_cal_init(g.nblk, o.t_lo, o.t_hi, ctx->lo, ctx->hi, ctx->ebar, ctx->ctl, ctx->s);
     CKL();
     const double inv_count = 1.0 / ((double)o.n_meas * (double)chains);
-    cluster_calibration(ctx);   // (asks the device outside any capture)
+    TRY(prepare_resident(ctx));   // (asks the device outside any capture)
     launch_fill_samples(g, ctx->mask, ctx->dang, ctx->ang, MPR_STORE_F32, ctx->Rp / 2, ctx->s);
     CKL();
     // auto and 1: graph; 2: persistent; 3: a launch per kernel from the host.
@@ -1820,6 +1914,13 @@ mpr_status mpr_calibrate(mpr_ctx* ctx, float* block_T_out) {
         launch_cal_fill(ctx->sl, g.nbx, ctx->Nsp_cal, ctx->T, ctx->beta, ctx->s);
         CKL();
     }
+    if (ctx->resident) {
+        uint32_t error = 0;
+        CK(cudaMemcpyAsync(&error, ctx->res_sync, sizeof(error), cudaMemcpyDeviceToHost, ctx->s));
+        CK(cudaStreamSynchronize(ctx->s));
+        if (error)
+            return fail(ctx, MPR_ETIMEOUT, "calibration: a wait between CTAs gave up (%u)", error);
+    }
     const int64_t cal_sweeps =
         o.n_bisect <= 0 ? 0
         : o.cal_continue < 0 ? (int64_t)o.n_bisect * (o.n_eq + o.n_meas)
@@ -1832,6 +1933,21 @@ mpr_status mpr_calibrate(mpr_ctx* ctx, float* block_T_out) {
     CK(cudaStreamSynchronize(ctx->s));
     collect_events(ctx);
     return MPR_OK;
+}
+
+mpr_status mpr_calibrate(mpr_ctx* ctx, float* block_T_out) {
+    PhaseRange phase_range("mpr_calibrate");
+    if (!ctx) return MPR_EINVAL;
+    mpr_status st = calibrate(ctx, block_T_out);
+    // Where the resident form could not run to its end (a refused launch, a
+    // wait that gave up), the half-steps are launched one by one.
+    if (ctx->resident && (st == MPR_ETIMEOUT || st == MPR_ECUDA)) {
+        ctx->res_refused = true;
+        cudaGetLastError();
+        collect_events(ctx);
+        st = calibrate(ctx, block_T_out);
+    }
+    return st;
 }
 
 mpr_status mpr_sim_begin(mpr_ctx* ctx, int32_t n) {

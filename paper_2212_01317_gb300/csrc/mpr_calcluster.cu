@@ -46,22 +46,6 @@ __device__ __forceinline__ void cluster_wait() {
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// Sum of a pair's weighted changes as an unevaluated sum hi + lo.
-struct Sum2 {
-    float2 hi, lo;
-    __device__ void add(float2 x, float w) {
-        const float2 w2 = both(w);
-        const float2 p = __fmul2_rn(x, w2);
-        const float2 e = __ffma2_rn(x, w2, make_float2(-p.x, -p.y));        // x w = p + e
-        const float2 s = __fadd2_rn(hi, p);
-        const float2 t = __ffma2_rn(hi, both(-1.0f), s);
-        const float2 a = __ffma2_rn(__ffma2_rn(t, both(-1.0f), s), both(-1.0f), hi);
-        const float2 b = __ffma2_rn(t, both(-1.0f), p);                     // hi + p = s + a + b
-        lo = __fadd2_rn(lo, __fadd2_rn(__fadd2_rn(a, b), e));
-        hi = s;
-    }
-};
-
 // A cell: (cos, sin) of q phi in the pair's even, then its odd realization.
 // Cells of a CTA: one per owned site and colour, then four per thread for the
 // neighbours that are not gap sites.

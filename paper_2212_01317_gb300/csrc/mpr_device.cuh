@@ -127,6 +127,22 @@ __device__ __forceinline__ float2 atan2_upper_2(float2 S, float2 C) {
     return make_float2(C.x < 0.0f ? g.x : a.x, C.y < 0.0f ? g.y : a.y);
 }
 
+// Sum of a pair's weighted changes as an unevaluated sum hi + lo.
+struct Sum2 {
+    float2 hi, lo;
+    __device__ void add(float2 x, float w) {
+        const float2 w2 = both(w);
+        const float2 p = __fmul2_rn(x, w2);
+        const float2 e = __ffma2_rn(x, w2, make_float2(-p.x, -p.y));        // x w = p + e
+        const float2 s = __fadd2_rn(hi, p);
+        const float2 t = __ffma2_rn(hi, both(-1.0f), s);
+        const float2 a = __ffma2_rn(__ffma2_rn(t, both(-1.0f), s), both(-1.0f), hi);
+        const float2 b = __ffma2_rn(t, both(-1.0f), p);                     // hi + p = s + a + b
+        lo = __fadd2_rn(lo, __fadd2_rn(__fadd2_rn(a, b), e));
+        hi = s;
+    }
+};
+
 // Outcome of one site update: the new angle, the angle after the Metropolis
 // move, the energy change, and whether the over-relaxation was applied.
 struct SiteNew {

@@ -244,6 +244,28 @@ struct CalClusterArgs {
     double *ebar, *ebar_odd, *ebar_pts;   // as FoldArgs
 };
 
+// The same for fields of up to kCalResidentSites gap sites per colour and CTA,
+// a group of CTAs of one cooperative launch per realization pair
+// (mpr_calresident.cu).
+constexpr int kCalResidentThreads = 1024;
+constexpr int kCalResidentSites = 2 * kCalResidentThreads;
+constexpr int kCalResidentCtas = 256;      // CTAs per pair at most
+struct CalResidentPlan {       // over the CTAs of a pair, each the largest
+    int most, consts, edges, blocks;   // most: sites of a colour
+    int sites;                         // of both, each in whole warps
+};
+struct CalResidentArgs {
+    CalClusterArgs cal;
+    const int* part;           // [2][ctas + 1] first list entry of each CTA, by colour
+    int ctas;                  // per pair
+    int cap;                   // sites of a colour at most (a multiple of 32)
+    int sites, halo, consts, edges, blocks;   // shared-memory capacities
+    uint32_t* sync;            // [0] error, [1] arrivals
+    float4* exports;           // [pairs][ctas][2][cap] angles that other CTAs read (zeroed)
+    uint32_t arrivals;         // arrivals awaited at the start
+    uint32_t spin_limit;       // polls
+};
+
 // Grid-wide barrier state of a cooperative launch (zeroed before each launch).
 struct GridBarrier {
     unsigned int arrive;   // CTAs arrived at the current barrier

@@ -174,6 +174,13 @@ void launch_sweep_tile(const SweepArgs& a, int storage, int grid, cudaStream_t s
 // the GPU at once (0: not available), and the launch.
 int cal_cluster_max_active();
 cudaError_t launch_cal_cluster(const CalClusterArgs& a, cudaStream_t s);
+// The resident form (mpr_calresident.cu). plan: part [2][ctas + 1] and the
+// largest needs of a CTA, as CalResidentPlan in `res` (zeroed by the call).
+void launch_cal_resident_plan(const uint4* const list[2], const int32_t* const start[2],
+                              const int64_t n[2], int ctas, int* part, int* res, cudaStream_t s);
+size_t cal_resident_smem_max(int device);   // bytes of dynamic shared memory, 0: unusable
+size_t cal_resident_smem(const CalResidentArgs& a);
+cudaError_t launch_cal_resident(const CalResidentArgs& a, cudaStream_t s);
 
 int cal_persistent_blocks_per_sm(int G);
 cudaError_t launch_cal_persistent(const CalPersistArgs& a, int G, int grid, cudaStream_t s);

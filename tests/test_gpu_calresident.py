@@ -1,0 +1,106 @@
+"""Calibration by resident CTAs (one cooperative launch per iteration) against a
+launch per half-step on the same chains.
+
+cal_sweep = 1 forces the launches; the automatic choice takes the resident form
+beyond 8192 gap sites per colour while the field's sites fit the shared memory
+of the GPU. Both run the same moves on the same random numbers and form the
+same FP32 warp sums; what lies above a warp is summed in another order. A
+bracket step decides differently only where a block's mean energy and e_s agree
+within that rounding, about 1e-8 against spreads of 1e-2: 1e-6 per decision. So
+of the at most 1e5 decisions of a case here none is expected to differ; two
+blocks' temperatures are allowed to.
+"""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_2212_01317_gb300 import synth
+from paper_2212_01317_gb300.mpr import BatchFiller, GapFiller
+
+pytestmark = pytest.mark.gpu
+
+OPTS = dict(seed=31, n_bisect=5, n_eq=5, n_meas=4)
+
+
+def _temperatures(z, m, lb, **opts):
+    v = np.where(m != 0, np.nan, z).astype(np.float32)
+    out = []
+    for form in (0, 1):
+        gf = GapFiller(v, m, lb, cal_sweep=form, **{**OPTS, **opts})
+        out.append(gf.calibrate())
+        gf.simulate(2)      # the context is usable afterwards
+        gf.close()
+    return out
+
+
+# just past the cluster form, partial warps and blocks, tiny and large blocks,
+# nearly all sites missing (few samples) and few of them (samples all around),
+# the largest field with every second site missing, one past the capacity
+@pytest.mark.parametrize("h,w,lb,p", [(131, 129, 16, 0.99), (301, 157, 7, 0.6), (200, 333, 2, 0.5),
+                                      (640, 512, 64, 0.35), (900, 1100, 16, 0.12),
+                                      (500, 300, 16, 0.95), (1024, 1024, 16, 0.5),
+                                      (1201, 1180, 16, 0.5), (3, 9000, 8, 0.8)])
+@pytest.mark.parametrize("opts", [{}, {"cal_points": 2}, {"cal_points": 4, "cal_chains": 3, "init": 1},
+                                  {"cal_chains": 3, "q": 0.37}])
+def test_resident_form_equals_launch_form(h, w, lb, p, opts):
+    z, _ = synth.small_problem(h, w, 0.5, seed=h * w)
+    m = (np.random.default_rng(h + w).random((h, w)) < p).astype(np.uint8)
+    m[0, :2] = 0
+    a, b = _temperatures(z, m, lb, **opts)
+    assert np.count_nonzero(a != b) <= 2
+
+
+# colour 0 starts late in the block order (its first blocks hold no gap), and
+# colour 1 only in a few blocks
+@pytest.mark.parametrize("late", [0, 1])
+def test_lists_that_differ_in_extent(late):
+    z, m = synth.small_problem(256, 300, 0.6, seed=4)
+    y, x = np.mgrid[:256, :300]
+    rows = y < 128 if late == 0 else y >= 40
+    m[rows & ((y + x) % 2 == late)] = 0
+    a, b = _temperatures(z, m, 16, cal_points=2)
+    assert np.count_nonzero(a != b) <= 2
+
+
+def test_resident_form_of_a_batch():
+    zs, ms = zip(*(synth.small_problem(h, w, 0.5, seed=h) for h, w in ((131, 220), (224, 124), (99, 340))))
+    vs = [np.where(m != 0, np.nan, z).astype(np.float32) for z, m in zip(zs, ms)]
+    got = []
+    for form in (0, 1):
+        bf = BatchFiller(vs, list(ms), 8, cal_points=2, cal_sweep=form, **OPTS)
+        got.append(bf.calibrate())
+        bf.close()
+    assert np.count_nonzero(got[0] != got[1]) <= 2
+
+
+def test_a_wait_that_gives_up_falls_back_to_launches():
+    """The start waits for one arrival too many (barrier_test) for 20 ms: every
+    CTA returns, and the calibration runs with a launch per half-step."""
+    z, m = synth.small_problem(256, 256, 0.5, seed=8)
+    a, b = _temperatures(z, m, 16, barrier_test=1, wait_ms=20)
+    assert np.count_nonzero(a != b) <= 2
+
+
+def test_two_threads_at_once():
+    """Two contexts calibrate on streams of their own at the same time, several
+    times: each takes the whole GPU for a launch, and neither hinders the other."""
+    import torch
+
+    z, m = synth.small_problem(300, 280, 0.5, seed=9)
+    v = np.where(m != 0, np.nan, z).astype(np.float32)
+    out = [None, None]
+
+    def work(k):
+        stream = torch.cuda.Stream()
+        for _ in range(3):
+            gf = GapFiller(v, m, 16, cuda_stream=stream.cuda_stream, **OPTS)
+            out[k] = gf.calibrate()
+            gf.close()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert np.count_nonzero(out[0] != out[1]) <= 2
