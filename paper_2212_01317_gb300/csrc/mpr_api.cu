@@ -932,9 +932,16 @@ mpr_status prepare_resident(mpr_ctx* ctx) {
     if (ctas < 1 || most > (int64_t)ctas * kCalResidentSites) return MPR_OK;
     const size_t smem = cal_resident_smem_max(ctx->device);
     if (smem == 0) return MPR_OK;
+    // (the launches need none of its memory)
+    auto no_memory = [ctx] {
+        ctx->err.clear();
+        return MPR_OK;
+    };
     constexpr size_t kPart = 2 * (kCalResidentCtas + 1);
     if (ctx->res_ctas != ctas) {
-        if (!ctx->res_part) TRY(dalloc(ctx, &ctx->res_part, kPart + sizeof(CalResidentPlan) / 4));
+        if (!ctx->res_part &&
+            dalloc(ctx, &ctx->res_part, kPart + sizeof(CalResidentPlan) / 4) != MPR_OK)
+            return no_memory();
         ctx->res_ctas = 0;
         launch_cal_resident_plan(ctx->list, ctx->start, ctx->n_gap, ctas, ctx->res_part,
                                  ctx->res_part + kPart, ctx->s);
@@ -965,7 +972,7 @@ mpr_status prepare_resident(mpr_ctx* ctx) {
         dfree(ctx, ctx->res_sync);
         ctx->res_sync = nullptr;
         ctx->res_cap = 0;
-        TRY(dalloc(ctx, &ctx->res_sync, need));
+        if (dalloc(ctx, &ctx->res_sync, need) != MPR_OK) return no_memory();
         ctx->res_cap = need;
     }
     CK(cudaMemsetAsync(ctx->res_sync, 0, sizeof(uint32_t), ctx->s));

@@ -16,7 +16,7 @@ import numpy as np
 import pytest
 
 from paper_2212_01317_gb300 import synth
-from paper_2212_01317_gb300.mpr import BatchFiller, GapFiller
+from paper_2212_01317_gb300.mpr import MPR_ENOMEM, BatchFiller, GapFiller, MprError
 
 pytestmark = pytest.mark.gpu
 
@@ -104,3 +104,28 @@ def test_two_threads_at_once():
     for t in threads:
         t.join()
     assert np.count_nonzero(out[0] != out[1]) <= 2
+
+
+def test_a_refused_workspace_falls_back_to_launches():
+    """Any allocation of a calibration may be refused (alloc_test): those only the
+    resident form needs leave the launches, the others end the call, and a second
+    call succeeds. The temperatures are the same."""
+    z, m = synth.small_problem(256, 256, 0.5, seed=8)
+    v = np.where(m != 0, np.nan, z).astype(np.float32)
+    want, _ = _temperatures(z, m, 16)
+    runs = 0
+    for k in range(1, 60):
+        try:
+            gf = GapFiller(v, m, 16, alloc_test=k, **OPTS)
+        except MprError as e:
+            assert e.status == MPR_ENOMEM
+            continue
+        try:
+            got = gf.calibrate()
+            runs += 1
+        except MprError as e:
+            assert e.status == MPR_ENOMEM
+            got = gf.calibrate()
+        gf.close()
+        assert np.count_nonzero(got != want) <= 2
+    assert runs >= 2
