@@ -672,14 +672,14 @@ def run_ours(args, world, rank, local):
         "frac": (achieved / peak) if achieved else None, "traffic": traffic,
         "kernel": ("k_sweep_half / k_sweep (realizations' per-launch half-steps)" if dom == "sim"
                    else ("k_sweep_flat (calibration)" if args.cal_mode == 3
-                         else "calibration graph (k_sweep_flat + bookkeeping)")),
+                         else "calibration graph (its iterations' sweeps + bookkeeping)")),
         "peak_kind": peak_kind,
         "bytes_per_gap_update": bpu,
         "avg_launch_us": 1e3 * (sim_ms / sim_launch if dom == "sim" else cal_ms / max(cal_launch, 1)),
         "sim_halfstep": {"ms": sim_ms / args.steps, "launches": sim_launch // args.steps,
                          "gbs": sim_gbs,
                          "updates_per_s": sweep_updates / (sim_ms / 1e3) if sim_ms else None},
-        "stop_tail": {"kernel": "k_pair_tail (one CTA per realization pair; its time includes "
+        "stop_tail": {"kernel": "k_pair_tail (a cluster per realization pair; its time includes "
                                 "the stop tests of its sweeps)",
                       "ms": tail_ms / args.steps, "launches": tail_launch // args.steps,
                       "updates": tail_updates // args.steps,

@@ -406,7 +406,7 @@ mpr_status mpr_predict(mpr_ctx* ctx, float* out, const float* truth, double* aae
  *   1: G = 8, two units per warp (form 3);
  *   2: G = 8, the staged half-step on tiles of at most 16 x 32 sites (form 4);
  *   3: G = 2, one warp per unit (form 0).
- * G is the lane-group width (realizations interleaved per site). The results
+ * G is the lane-group width (the group option). The results
  * do not depend on the choice (the random streams are keyed by realization,
  * not by lane or form). The trial batches are discarded: nothing is
  * accumulated or counted. Needs temperatures; no batch may be open.
